@@ -561,8 +561,8 @@ def measure_variants(args):
     return out
 
 
-KRYLOV_SOURCES = ("csrc/krylov_impl.cuh", "csrc/krylov.cu", "csrc/operator.cuh", "csrc/common.cuh",
-                  "csrc/kernels.h")
+KRYLOV_SOURCES = ("csrc/krylov_impl.cuh", "csrc/krylov_mma.cuh", "csrc/krylov.cu", "csrc/operator.cuh",
+                  "csrc/common.cuh", "csrc/kernels.h")
 # DRAM bytes per launch of the Krylov kernel on the 1024^2 pair, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the
 # kernel sources whose SHA-256 is recorded with it.
@@ -850,7 +850,7 @@ def run_ours(args):
                        "mean_active_points": upd / max(1, args.steps * ws),
                        "l2": "flushed between timed steps (256 MiB write outside the step events)",
                        "wall_s": wall},
-            "roofline": {"bound": "hbm", "kernel": "k_krylov_step (Arnoldi, phi_1 and the update: the Krylov "
+            "roofline": {"bound": "hbm", "kernel": "k_krylov_mma (Arnoldi, phi_1 and the update: the Krylov "
                                                     "part of a step)",
                          "achieved": achieved_gbs, "peak": peak, "unit": "GB/s", "frac": achieved_gbs / peak,
                          "peak_source": f"{peak_src} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)",

@@ -124,6 +124,7 @@ struct wrc_run {
     DevBuf rows;        // NJ + 1 ints: flags of the row pairs of psi a step reads, their count and list
     bool rows_psi = false;   // psi of the last freeze holds only those rows
     long long cap_g = 0;
+    bool batched = false;    // stepped in batched launches: its basis is allocated with the grid
 
     // Krylov small arrays and cooperative-kernel scratch
     struct {
@@ -194,7 +195,7 @@ struct wrc_run {
     // launch: its own basis, work vector, ghost values, lattice vector,
     // partial sums and barrier words, and the launch's argument array and
     // block map (device, with a pinned host copy)
-    DevBuf sbasis, sw, sGb, sLq, spart, sbar, sdev;
+    DevBuf sbasis, sw, sus, sGb, sLq, spart, sbar, sdev;
     void* shost = nullptr;
     size_t shost_bytes = 0;
 
@@ -257,6 +258,16 @@ double* lattice_scratch(wrc_run* R) {
     return R->lat64.as<double>();
 }
 
+// The basis and its ghost values in global memory: for the batched and the
+// streaming Krylov launches and the Rosenbrock step (a single run's launch
+// keeps them in shared memory as long as they fit).
+wrc_status ensure_basis(wrc_run* R) {
+    const size_t m = R->cfg.krylov_m;
+    CK(R->basis.grow(8 * (size_t)R->cap * (m + 1), 0, R->st));   // 64-bit fixed point (or the bulk type)
+    CK(R->Gb.grow(8 * (size_t)R->cap_g * (m + 3), 0, R->st));
+    return WRC_OK;
+}
+
 wrc_status ensure_capacity(wrc_run* R, long long n) {
     if (n <= R->cap) return WRC_OK;
     long long c = n + n / 4 + 1024;
@@ -290,9 +301,9 @@ wrc_status ensure_capacity(wrc_run* R, long long n) {
     if (R->cfg.scheme == WRC_SCHEME_ROSENBROCK) CK(R->jac.grow(4 * be, 0, s));
     // the basis is rebuilt every step; its leading dimension changes with c
     R->basis.release(s);
-    CK(R->basis.grow(be * (size_t)(m + 1), 0, s));
     R->cap = c;
     R->layout += 1;
+    if (R->batched || R->cfg.scheme == WRC_SCHEME_ROSENBROCK) TRY(ensure_basis(R));
     return WRC_OK;
 }
 
@@ -301,15 +312,14 @@ wrc_status ensure_ghost_capacity(wrc_run* R, long long ng) {
     long long c = ng + ng / 4 + 1024;
     c = (c + 255) / 256 * 256;
     const cudaStream_t s = R->st;
-    const int m = R->cfg.krylov_m;
     CK(R->row_len.grow(sizeof(int) * c, 0, s));
     CK(R->row_ready.grow(sizeof(int) * (c + 1), 0, s));
     CK(R->row_idx.grow(sizeof(int) * c * R->rmax, 0, s));
     CK(R->row_w.grow(sizeof(double) * c * R->rmax, 0, s));
     R->Gb.release(s);
-    CK(R->Gb.grow(R->es * c * (m + 1), 0, s));
     R->cap_g = c;
     R->layout += 1;
+    if (R->batched || R->cfg.scheme == WRC_SCHEME_ROSENBROCK) TRY(ensure_basis(R));
     return WRC_OK;
 }
 
@@ -699,6 +709,7 @@ KrylovStepArgs krylov_args(wrc_run* R) {
     A.basis = R->basis.p;
     A.ld = R->cap;
     A.w = R->w.p;
+    A.us = R->tmp.p;
     A.H = R->K.H;
     A.y = R->K.y;
     A.beta = R->K.beta;
@@ -745,14 +756,12 @@ template <typename T>
 wrc_status krylov_pair(wrc_run* R, const KrylovStepArgs& A) {
     const cudaStream_t s = R->st;
     const int m = R->cfg.krylov_m;
-    constexpr int kPairPT = 128;   // threads per block of the batched kernel
-    const int maxb = krylov_batch_max_blocks(R->fp32, R->g.P, kPairPT, true);
-    if (maxb < 2) return fail(R, WRC_ERR_CUDA, "batched Krylov kernel occupancy query failed");
-    CK(R->sbasis.grow(R->es * (size_t)R->cap * (m + 1), 0, s));
+    CK(R->sbasis.grow(8 * (size_t)R->cap * (m + 1), 0, s));
     CK(R->sw.grow(R->es * (size_t)R->cap, 0, s));
-    CK(R->sGb.grow(R->es * (size_t)(R->cap_g > 0 ? R->cap_g : 1) * (m + 1), 0, s));
+    CK(R->sus.grow(R->es * (size_t)R->cap, 0, s));
+    CK(R->sGb.grow(8 * (size_t)(R->cap_g > 0 ? R->cap_g : 1) * (m + 3), 0, s));
     CK(R->sLq.grow(R->es * (size_t)R->N, 0, s));
-    CK(R->spart.grow(sizeof(double) * krylov_partials_doubles(maxb), 0, s));
+    CK(R->spart.grow(sizeof(double) * krylov_partials_doubles(), 0, s));
     if (!R->sbar.p) {
         CK(R->sbar.grow(sizeof(unsigned) * 4, 0, s));
         CK(cudaMemsetAsync(R->sbar.p, 0, R->sbar.bytes, s));
@@ -760,14 +769,15 @@ wrc_status krylov_pair(wrc_run* R, const KrylovStepArgs& A) {
     KrylovStepArgs B = krylov_args_scalar(R);
     B.basis = R->sbasis.p;
     B.w = R->sw.p;
+    B.us = R->sus.p;
     B.Gb = R->sGb.p;
     B.Lq = R->sLq.p;
     B.part = R->spart.as<double>();
     B.bar = R->sbar.as<unsigned>();
-    const long long need = (R->n_active + kPairPT - 1) / kPairPT;
-    const int each = (int)std::max(1LL, std::min(need, (long long)(maxb / 2)));
-    const int total = 2 * each;
-    const size_t bytes = 2 * sizeof(KrylovStepArgs) + sizeof(int) * (total + 3);
+    std::vector<int> items, off;
+    krylov_batch_plan({R->n_active, R->n_active}, 128, R->max_blocks, items, off);
+    const int total = (int)off.size() - 1;
+    const size_t bytes = 2 * sizeof(KrylovStepArgs) + sizeof(int) * (items.size() + off.size());
     CK(R->sdev.grow(bytes, 0, s));
     if (R->shost_bytes < bytes) {
         CK(cudaStreamSynchronize(s));   // the last copy from the old staging buffer
@@ -780,17 +790,19 @@ wrc_status krylov_pair(wrc_run* R, const KrylovStepArgs& A) {
     KrylovStepArgs* ha = (KrylovStepArgs*)R->shost;
     ha[0] = A;
     ha[1] = B;
-    int* blk = (int*)(ha + 2);
-    for (int b = 0; b < total; ++b) blk[b] = b < each ? 0 : 1;
-    blk[total] = 0;
-    blk[total + 1] = each;
-    blk[total + 2] = total;
-    if (R->tracing) R->trace_nb = each;
+    int* hi = (int*)(ha + 2);
+    std::copy(items.begin(), items.end(), hi);
+    std::copy(off.begin(), off.end(), hi + items.size());
+    if (R->tracing) R->trace_nb = items[2];
     CK(cudaMemcpyAsync(R->sdev.p, R->shost, bytes, cudaMemcpyHostToDevice, s));
     const KrylovStepArgs* da = (const KrylovStepArgs*)R->sdev.p;
-    const int* dblk = (const int*)(da + 2);
-    CK(launch_krylov_batch<T>(da, dblk, dblk + total, 2, total, kPairPT, R->g.P, s, true));
+    const int* di = (const int*)(da + 2);
+    CK(launch_krylov_batch<T>(da, di, di + items.size(), total, R->g.P, s));
     return WRC_OK;
+}
+
+KrylovPlan krylov_plan_of(const wrc_run* R) {
+    return krylov_plan(R->n_active, R->n_ghost, R->cfg.krylov_m, R->fp32, R->g.P, R->device, R->cluster_max);
 }
 
 // Clear the phase trace before a traced launch (on the run's stream).
@@ -811,9 +823,11 @@ wrc_status krylov(wrc_run* R) {
     const cudaStream_t s = R->st;
     const long long n = R->n_active;
     const int m = R->cfg.krylov_m;
+    const KrylovPlan plan = krylov_plan_of(R);
+    const bool pair = R->scalar && R->cfg.scheme != WRC_SCHEME_ROSENBROCK;
+    if (pair || plan.form == 3) TRY(ensure_basis(R));
     const KrylovStepArgs A = krylov_args(R);
-    const int blocks = krylov_step_blocks(n, R->max_blocks, R->fp32, R->g.P, R->device, R->cluster_max);
-    TRY(trace_reset(R, blocks));
+    TRY(trace_reset(R, plan.blocks));
     int e0 = -1;
     if (R->profiling) {
         while (R->ev_pool.size() < R->ev_used.size() * 2 + 2) {
@@ -824,16 +838,15 @@ wrc_status krylov(wrc_run* R) {
         e0 = (int)R->ev_used.size() * 2;
         CK(cudaEventRecord(R->ev_pool[e0], s));
     }
-    const bool pair = R->scalar && R->cfg.scheme != WRC_SCHEME_ROSENBROCK;
     if (R->cfg.scheme == WRC_SCHEME_ROSENBROCK) TRY(krylov_rosenbrock<T>(R));
     else if (pair) TRY(krylov_pair<T>(R, A));
-    else CK(launch_krylov_step<T>(A, blocks, s, R->device, R->cluster_max));
+    else CK(launch_krylov_step<T>(A, plan, s, R->device));
     if (R->profiling) {
         CK(cudaEventRecord(R->ev_pool[e0 + 1], s));
         const double f = pair ? 2.0 : 1.0;
         R->ev_used.push_back({e0, f * krylov_algorithmic_bytes(n, m), f * krylov_algorithmic_flops(n, m)});
     }
-    if (R->scalar && !pair) CK(launch_krylov_step<T>(krylov_args_scalar(R), blocks, s, R->device, R->cluster_max));
+    if (R->scalar && !pair) CK(launch_krylov_step<T>(krylov_args_scalar(R), plan, s, R->device));
     return WRC_OK;
 }
 
@@ -1259,7 +1272,7 @@ void free_run(wrc_run* R) {
                     &R->basis, &R->tmp, &R->row_len, &R->row_ready, &R->row_idx, &R->row_w, &R->Gb, &R->lat64,
                     &R->trace, &R->rows, &R->rv[0],
                     &R->rv[1], &R->Lr, &R->kr, &R->jac, &R->rbpart, &R->rbsmall, &R->pe[0], &R->pe[1], &R->Lp, &R->Lqx,
-                    &R->xd, &R->xbasis, &R->xw, &R->sbasis, &R->sw, &R->sGb, &R->sLq, &R->spart, &R->sbar, &R->sdev})
+                    &R->xd, &R->xbasis, &R->xw, &R->sbasis, &R->sw, &R->sus, &R->sGb, &R->sLq, &R->spart, &R->sbar, &R->sdev})
         b->release(s);
     cudaStreamSynchronize(s);
     void* ptrs[] = {R->L, R->Lq, R->psi, R->C1, R->C2, R->act, R->nxt, R->gho, R->sig, R->JJ, R->halo, R->list, R->lat2idx,
@@ -1371,8 +1384,7 @@ wrc_status wrc_create(const wrc_config* cfg, void* cuda_stream, wrc_run** out) {
     }
     if (e == cudaSuccess) e = alloc((void**)&R->K.H, sizeof(double) * ((m + 1) * m + 1 + 32));
     if (e == cudaSuccess) e = alloc((void**)&R->K.kstop, sizeof(int) * 8);
-    const size_t npart = krylov_partials_doubles(R->max_blocks) > (size_t)kMaxBlocks * 4
-                             ? krylov_partials_doubles(R->max_blocks) : (size_t)kMaxBlocks * 4;
+    const size_t npart = std::max(krylov_partials_doubles(), (size_t)kMaxBlocks * 4);
     if (e == cudaSuccess) e = alloc((void**)&R->K.part, sizeof(double) * npart);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&R->counts_host, sizeof(int) * (kMaxKeys + 4));
     if (e != cudaSuccess) {
@@ -1790,7 +1802,7 @@ wrc_status wrc_profile(wrc_run* R, int32_t enable) {
 
 wrc_status wrc_query_krylov_form(wrc_run* R, int32_t* cluster_size) {
     if (!R || !cluster_size) return WRC_ERR_ARG;
-    *cluster_size = krylov_step_cluster(R->n_active, R->max_blocks, R->fp32, R->g.P, R->device, R->cluster_max);
+    *cluster_size = krylov_plan_of(R).cluster;
     return WRC_OK;
 }
 
@@ -1890,39 +1902,26 @@ wrc_status cfail(BatchCtx& C, wrc_status s, const std::string& msg) {
                          std::string(#call) + ": " + cudaGetErrorString(e_));                   \
     } while (0)
 
-// Block plan: run i gets ceil(n_i / (pt * ept)) blocks, clamped to
-// [1, its partial-sum capacity]; if the total exceeds what can be co-resident,
-// every run's share is scaled down (keeping at least one block each).
-wrc_status plan_batch(BatchCtx& C, const std::vector<wrc_run*>& runs, int max_coresident, int& total) {
+// Block plan (krylov_batch_plan): a run gets another block of the launch while
+// its share stays above pt * ept points, the block shape's tile.
+wrc_status plan_batch(BatchCtx& C, const std::vector<wrc_run*>& runs, int& total, int& nitems) {
     const size_t M = runs.size();
-    std::vector<int> nb(M);
-    long long sum = 0;
-    for (size_t i = 0; i < M; ++i) {
-        const wrc_run* R = runs[i];
-        long long b = (R->n_active + (long long)C.pt * C.ept - 1) / ((long long)C.pt * C.ept);
-        b = b < 1 ? 1 : b;
-        b = b > R->max_blocks ? R->max_blocks : b;
-        nb[i] = (int)b;
-        sum += b;
-    }
-    if ((long long)M > max_coresident)
+    if ((long long)M > krylov_batch_max_runs(C.pt))
         return cfail(C, WRC_ERR_ARG, "more runs than co-resident blocks of the batched kernel");
-    if (sum > max_coresident) {
-        const double f = (double)(max_coresident - (long long)M) / (double)(sum - (long long)M);
-        sum = 0;
-        for (size_t i = 0; i < M; ++i) {
-            nb[i] = 1 + (int)std::floor((nb[i] - 1) * f);
-            sum += nb[i];
-        }
-    }
-    total = (int)sum;
-    if (total + (int)M + 1 > C.blk_cap) {
+    std::vector<long long> n(M);
+    for (size_t i = 0; i < M; ++i) n[i] = runs[i]->n_active;
+    std::vector<int> items, off;
+    krylov_batch_plan(n, (long long)C.pt * C.ept, runs[0]->max_blocks, items, off);
+    total = (int)off.size() - 1;
+    nitems = (int)items.size();
+    const int need = (int)(items.size() + off.size());
+    if (need > C.blk_cap) {
         BCK(cudaStreamSynchronize(C.main));   // the old tables may still be read
         if (C.h_blk) cudaFreeHost(C.h_blk);
         if (C.d_blk) cudaFree(C.d_blk);
         C.h_blk = nullptr;
         C.d_blk = nullptr;
-        C.blk_cap = total + (int)M + 1 + 1024;
+        C.blk_cap = need + 1024;
         BCK(cudaMallocHost((void**)&C.h_blk, sizeof(int) * C.blk_cap));
         BCK(cudaMalloc((void**)&C.d_blk, sizeof(int) * C.blk_cap));
     }
@@ -1936,15 +1935,8 @@ wrc_status plan_batch(BatchCtx& C, const std::vector<wrc_run*>& runs, int max_co
         BCK(cudaMallocHost((void**)&C.h_args, sizeof(KrylovStepArgs) * C.args_cap));
         BCK(cudaMalloc((void**)&C.d_args, sizeof(KrylovStepArgs) * C.args_cap));
     }
-    int* blk2mem = C.h_blk;
-    int* b0 = C.h_blk + total;
-    int off = 0;
-    for (size_t i = 0; i < M; ++i) {
-        b0[i] = off;
-        for (int b = 0; b < nb[i]; ++b) blk2mem[off + b] = (int)i;
-        off += nb[i];
-    }
-    b0[M] = off;
+    std::copy(items.begin(), items.end(), C.h_blk);
+    std::copy(off.begin(), off.end(), C.h_blk + items.size());
     return WRC_OK;
 }
 
@@ -1955,32 +1947,27 @@ wrc_status batch_krylov(BatchCtx& C, const std::vector<wrc_run*>& live) {
         BCK(cudaEventRecord(C.ev_streams[q], C.streams[q]));
         BCK(cudaStreamWaitEvent(C.main, C.ev_streams[q], 0));
     }
-    const int maxb = krylov_batch_max_blocks(C.fp32, C.P, C.pt);
-    if (maxb <= 0) return cfail(C, WRC_ERR_CUDA, "batched Krylov kernel occupancy query failed");
-    int total = 0;
-    TRY(plan_batch(C, live, maxb, total));
+    int total = 0, nitems = 0;
+    TRY(plan_batch(C, live, total, nitems));
     const size_t M = live.size();
-    int max_n = 1;
     for (size_t i = 0; i < M; ++i) {
         C.h_args[i] = krylov_args(live[i]);
-        max_n = std::max(max_n, (int)live[i]->n_active);
         if (live[i]->tracing) {
-            const int nbi = C.h_blk[total + i + 1] - C.h_blk[total + i];
             wrc_run* R = live[i];
-            R->trace_nb = nbi;
+            for (int q = 0; q < nitems; q += 3)
+                if (C.h_blk[q] == (int)i) R->trace_nb = C.h_blk[q + 2];
             BCK(cudaMemsetAsync(R->trace.p, 0, R->trace.bytes, C.main));
         }
     }
     BCK(cudaMemcpyAsync(C.d_args, C.h_args, sizeof(KrylovStepArgs) * M, cudaMemcpyHostToDevice, C.main));
-    BCK(cudaMemcpyAsync(C.d_blk, C.h_blk, sizeof(int) * (total + M + 1), cudaMemcpyHostToDevice, C.main));
+    BCK(cudaMemcpyAsync(C.d_blk, C.h_blk, sizeof(int) * (nitems + total + 1), cudaMemcpyHostToDevice, C.main));
     cudaEvent_t pa = nullptr, pb = nullptr;
     if (C.profiling) {
         BCK(cudaEventCreate(&pa));
         BCK(cudaEventCreate(&pb));
         BCK(cudaEventRecord(pa, C.main));
     }
-    (void)max_n;
-    BCK(launch_krylov_batch<T>(C.d_args, C.d_blk, C.d_blk + total, (int)M, total, C.pt, C.P, C.main));
+    BCK(launch_krylov_batch<T>(C.d_args, C.d_blk, C.d_blk + nitems, total, C.P, C.main));
     if (C.profiling) {
         BCK(cudaEventRecord(pb, C.main));
         C.prof.push_back({pa, pb});
@@ -2178,6 +2165,8 @@ void wrc::store_tuned_shape(bool fp32, long long runs, long long active, int pt,
     g_tune_cache[{fp32, log2_bucket(runs), log2_bucket(active)}] = {pt, ept};
 }
 
+void wrc::mark_batched(wrc_run* R) { R->batched = true; }
+
 double wrc::run_bytes_for(const wrc_config& cfg, long long na, long long ng) {
     const double N = (double)((long long)cfg.n0 << cfg.J) * (double)((long long)cfg.n0 << cfg.J);
     const double es = cfg.prec == WRC_MIXED ? 4.0 : 8.0;
@@ -2191,12 +2180,12 @@ double wrc::run_bytes_for(const wrc_config& cfg, long long na, long long ng) {
     b += 4.0 * es * std::sqrt(N) + 16.0 * std::sqrt(N);
     // Krylov small arrays and partial sums (at most kMaxBlocks blocks)
     b += 8.0 * (m1 * cfg.krylov_m + 33) +
-         8.0 * (double)std::max(krylov_partials_doubles(kMaxBlocks), (size_t)kMaxBlocks * 4);
+         8.0 * (double)std::max(krylov_partials_doubles(), (size_t)kMaxBlocks * 4);
     const double c = (double)grown_capacity(na), cg = (double)grown_capacity(ng);
     // meta x2, omega x2, details, U, V, g, w, basis (m+1), doubles scratch
-    b += c * (8.0 + 2.0 * es + 5.0 * es + es * m1 + 8.0);
+    b += c * (8.0 + 2.0 * es + 5.0 * es + 8.0 * m1 + 8.0);
     // ghost rows: length, ready flag, dd_row_max(p) indices and weights; ghost basis values
-    b += cg * (8.0 + (4.0 + 8.0) * dd_row_max(cfg.p == 0 ? 2 : cfg.p) + es * m1) + 4.0;
+    b += cg * (8.0 + (4.0 + 8.0) * dd_row_max(cfg.p == 0 ? 2 : cfg.p) + 8.0 * (m1 + 2.0)) + 4.0;
     return b;
 }
 
@@ -2209,7 +2198,7 @@ double wrc::run_device_bytes(const wrc_run* R) {
     double b = 7.0 * es * N + 6.0 * N + 8.0 * N + 8.0 * nblk * kMaxKeys + (double)R->lat64.bytes;
     b += 4.0 * es * R->g.NJ + 16.0 * R->g.NJ;
     b += 8.0 * (m1 * cfg.krylov_m + 33) +
-         8.0 * (double)std::max(krylov_partials_doubles(R->max_blocks), (size_t)kMaxBlocks * 4);
+         8.0 * (double)std::max(krylov_partials_doubles(), (size_t)kMaxBlocks * 4);
     const DevBuf* bufs[] = {&R->meta[0], &R->meta[1], &R->omega[0], &R->omega[1], &R->Ua, &R->Va, &R->ga,
                             &R->det, &R->w, &R->basis, &R->tmp, &R->row_len, &R->row_ready, &R->row_idx, &R->row_w,
                             &R->Gb, &R->rows};
@@ -2283,6 +2272,7 @@ wrc_status wrc_ensemble_create(int32_t n, const wrc_config* cfgs, void* cuda_str
         wrc_run* R = nullptr;
         const wrc_status st = wrc_create(&cfgs[i], E->C.streams[i % S], &R);
         if (st != WRC_OK) return cleanup(st, "member " + std::to_string(i) + ": " + g_create_error);
+        mark_batched(R);
         E->members.push_back(R);
     }
     *out = E;
@@ -2342,7 +2332,7 @@ wrc_status wrc_ensemble_tune(wrc_ensemble* E, int32_t steps_per_candidate, int32
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) {
             // a shape needs one co-resident block per member at least
-            if (krylov_batch_max_blocks(E->C.fp32, E->C.P, pts[a]) < (int)E->members.size()) continue;
+            if (krylov_batch_max_runs(pts[a]) < (int)E->members.size()) continue;
             E->C.pt = pts[a];
             E->C.ept = epts[b];
             E->C.profiling = true;

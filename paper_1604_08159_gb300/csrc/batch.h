@@ -60,6 +60,10 @@ double batch_take_profile(BatchCtx& C);
 bool tuned_shape(bool fp32, long long runs, long long active, int& pt, int& ept);
 void store_tuned_shape(bool fp32, long long runs, long long active, int pt, int ept);
 
+// Tells a new run, before its initial condition, that it is stepped in
+// batched launches.
+void mark_batched(wrc_run* R);
+
 // The checks wrc_create makes on a configuration (why explains a failure).
 bool valid_run_config(const wrc_config* cfg, std::string& why);
 

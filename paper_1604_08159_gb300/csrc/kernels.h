@@ -1,6 +1,8 @@
 // Host-side launchers of the library's CUDA kernels (internal interface).
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 
 namespace wrc {
@@ -230,7 +232,7 @@ struct KrylovStepArgs {
     const double* row_w;
     int rmax;
     const int* row_overflow; // non-zero: some row exceeded rmax (the kernel refuses to run)
-    void* Gb;               // ghost values of the basis vectors, (m+1) x ldg
+    void* Gb;               // streaming form: ghost values of the basis vectors, (m+3) x ldg 64-bit words
     long long ldg;
     // arrays of the run's bulk type (double, or float for the mixed mode)
     const void* Ua;
@@ -240,15 +242,16 @@ struct KrylovStepArgs {
     void* L;                // R(omega) on the lattice (in), omega^{n+1} at the active points (out)
     void* Lq;               // lattice array of the current Krylov vector and its ghost values
     void* omega;            // compact omega, updated in place
-    void* basis;            // (m+1) x ld
+    void* basis;            // streaming form: (m+1) x ld 64-bit words
     long long ld;
-    void* w;
+    void* w;                // z = A u at the active points, read through the ghosts' rows
+    void* us;               // u at the active points (streaming form)
     double* H;              // (m+1) x m row-major
     double* y;              // m
     double* beta;           // [1]
     int* kstop;             // [1] Krylov dimension used
     int* flags;             // [1] bit 0: non-finite value met
-    double* part;           // 3 x blocks x 33 partial sums
+    double* part;           // grid-wide sums and exponents (krylov_partials_doubles)
     unsigned* bar;          // grid barrier: {count, generation}
     int* err;               // bit 1: a barrier wait ran out; bit 2 (4): row overflow; bit 4 (16): a clustered
                             // launch did not form its clusters and ran unclustered (not an error)
@@ -263,52 +266,57 @@ struct KrylovStepArgs {
     unsigned long long* trace;
 };
 constexpr int kTracePhases = 3 + 3 * 31;
-// Co-resident capacity of the single-run Krylov kernel on device dev (also
-// for clusters of 2 and 4 blocks, kept per device and precision for
-// krylov_step_blocks and the launch; a cluster size whose clusters a probe
-// launch does not see formed is not used).
+// Sets up the Krylov kernels of (bulk type, DD order) on device dev: shared
+// memory, co-resident capacity, whether clusters of four blocks form (a
+// probe launch at the device's first call).  *max_blocks: its SMs.
 int krylov_step_init(int dev, bool fp32, int P, int* max_blocks);
 // Largest cluster size a run created now may use: 4, or the cap set by the
-// environment variable WRC_KRYLOV_CLUSTER (1 or 2), read when called.
+// environment variable WRC_KRYLOV_CLUSTER (1 or 2: no clusters), read when called.
 int krylov_cluster_max();
 // A clustered Krylov launch on device dev ran unclustered (its clusters were
 // not formed): later launches on the device are planned without clusters.
 void krylov_clusters_unformed(int dev);
-// Blocks for n active points: one thread per point, capped at max_blocks,
-// padded to a whole number of 4- or 2-block clusters (at most cmax) where
-// that fits.
-int krylov_step_blocks(long long n, int max_blocks, bool fp32, int P, int dev, int cmax);
-// Cluster size (1, 2 or 4) of the launch krylov_step_blocks plans for n points.
-int krylov_step_cluster(long long n, int max_blocks, bool fp32, int P, int dev, int cmax);
-// Cooperative launch on device dev (current); clusters of 4 or 2 (<= cmax) blocks when
-// `blocks` is a multiple within their capacity (their blocks pre-add the dot
-// sums in distributed shared memory).  The first clustered launch per device
-// and precision synchronises `s` and, if the clusters were not formed,
-// switches them off for the device and launches again without them.
+// A planned single-run Krylov launch on device dev: forms 0-2 keep their
+// table in shared memory (krylov_mma.cuh: ppb points and gpb ghosts per
+// block, the interpolation rows of nrc of these), form 3 streams it
+// (krylov_stream.cuh); clusters of `cluster` blocks (<= cmax).
+struct KrylovPlan {
+    int form = 0;
+    int blocks = 1, cluster = 1, ppb = 0, gpb = 0, nrc = 0;
+    size_t smem = 0;
+};
+KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int dev, int cmax);
+// Cooperative launch on device dev (current).  The first clustered launch per
+// device synchronises `s` and, if the clusters were not formed (it then ran
+// unclustered), switches them off for the device.
 template <typename T>
-cudaError_t launch_krylov_step(const KrylovStepArgs& args, int blocks, cudaStream_t s, int dev, int cmax);
-size_t krylov_partials_doubles(int max_blocks);
-// Batched Krylov step: `members` problems (device array of arguments) in one
-// cooperative launch of `blocks` blocks of pt (64, 128 or 256) threads; block
-// b works on problem blk2mem[b], whose blocks are mem_b0[q] .. mem_b0[q+1]-1.
-// pair: the spill-free form for the two problems of one run (pt = 128).
-int krylov_batch_max_blocks(bool fp32, int P, int pt, bool pair = false);
+cudaError_t launch_krylov_step(const KrylovStepArgs& args, const KrylovPlan& plan, cudaStream_t s, int dev);
+size_t krylov_partials_doubles();
+// Batched Krylov step of several problems (device array of arguments) in one
+// cooperative launch of the streaming form: block b works on the items
+// d_off[b] .. d_off[b + 1] - 1, each (problem, block index in it, its
+// blocks).  krylov_batch_plan fills them for problems of n points on sms
+// blocks, a problem getting another block while each keeps `least` points;
+// krylov_batch_max_runs is the most runs a batch of block shape pt accepts.
+void krylov_batch_plan(const std::vector<long long>& n, long long least, int sms, std::vector<int>& items,
+                       std::vector<int>& off);
+int krylov_batch_max_runs(int pt);
 template <typename T>
-cudaError_t launch_krylov_batch(const KrylovStepArgs* d_args, const int* d_blk2mem, const int* d_mem_b0,
-                                int members, int blocks, int pt, int P, cudaStream_t s, bool pair = false);
+cudaError_t launch_krylov_batch(const KrylovStepArgs* d_args, const int* d_items, const int* d_off, int blocks, int P,
+                                cudaStream_t s);
 
 // The kernels of one bulk type T and DD half-order P (2, 3, 4), compiled per
-// order in krylov_pP.cu: occupancy of the single-run kernel, co-resident
-// capacity for clusters of CL = 2 or 4 blocks, the single-run launch with
-// clusters of cl blocks (1: plain cooperative launch), and the batched
-// kernel for pt threads per block (64, 128, 256; nullptr otherwise; with
-// pair, its spill-free form, pt = 128 only).
+// order in krylov_pP.cu: the single-run kernel with clusters of cl blocks in
+// a form, the streaming kernel for a batch and for one problem.
 template <typename T, int P>
 struct KrylovKernels {
-    cudaError_t occupancy(int* per);
-    int cluster_capacity(int CL);
-    cudaError_t launch(const KrylovStepArgs& args, int blocks, int cl, cudaStream_t s);
-    const void* batch_kernel(int pt, bool pair = false);
+    const void* mma_kernel(int cl, int form);
+    int mma_threads();
+    size_t mma_bytes(int form, int m, int ppb, int gpb, int nrc);
+    const void* stream_kernel();
+    const void* stream_one_kernel();
+    size_t stream_bytes();
+    cudaError_t launch(const KrylovStepArgs& args, const KrylovPlan& plan, cudaStream_t s);
 };
 extern template struct KrylovKernels<double, 2>;
 extern template struct KrylovKernels<float, 2>;

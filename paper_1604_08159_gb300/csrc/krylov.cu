@@ -1,20 +1,21 @@
-// Host side of the Krylov-projected step (Sec. 2.1): co-resident capacity
-// and thread-block clusters per device, the probe and check of cluster
-// formation, the launches of the single-run and batched kernels, dispatched
-// by bulk type and DD order (the kernels are compiled per DD order in
-// krylov_p2.cu, krylov_p3.cu and krylov_p4.cu from krylov_impl.cuh).
+// Host side of the Krylov-projected step (Sec. 2.1): shared-memory opt-in,
+// co-resident capacity and thread-block clusters per device, the probe and
+// check of cluster formation, the plans of the single-run and batched
+// launches, dispatched by bulk type and DD order (the kernels are compiled
+// per DD order in krylov_p2.cu, krylov_p3.cu and krylov_p4.cu from
+// krylov_mma.cuh and krylov_stream.cuh).
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cstdlib>
 #include <mutex>
+#include <numeric>
 
 #include "kernels.h"
 
 namespace wrc {
 
 namespace {
-constexpr int kPT = 128;      // threads per block of the single-run kernel
-constexpr int kOutP = 66;     // partial sums per block (as in krylov_impl.cuh)
 
 // Cluster formation check: launched with the attributes of the clustered
 // Krylov kernel (cooperative, clusters of CL blocks, grid of one cluster),
@@ -33,21 +34,20 @@ auto by_order(int P, F&& f) {
 }  // namespace
 
 namespace {
-// Per device: whether clusters of 2 and 4 blocks form on the launch path
-// (probe), whether a clustered launch has been checked, and per bulk type and
-// DD order the co-resident blocks of the single-run kernel for clusters of
-// 1, 2 and 4 blocks (0 where that cluster size cannot be launched
-// cooperatively or does not form).
 constexpr int kMaxDevices = 64;
-struct ClusterCaps {
+// Per device, bulk type and DD order: co-resident blocks (one per SM), in
+// clusters of four (0: not formed), and the dynamic shared memory a block of
+// the single-run kernel may take.
+struct MmaCaps {
     bool ready = false;
-    int cap[3] = {0, 0, 0};
+    int cap1 = 0, cap4 = 0;
+    size_t bytes = 0;
 };
 struct DeviceClusters {
+    MmaCaps mma[2][kMaxP + 1];               // [fp32][P]
     bool probed = false;
-    bool formed[3] = {true, false, false};   // [log2 CL]
-    bool checked = false;
-    ClusterCaps caps[2][kMaxP + 1];          // [fp32][P]
+    bool formed4 = false;                    // clusters of four form on the launch path
+    bool checked = false;                    // a clustered launch has been checked
 };
 DeviceClusters g_dev[kMaxDevices];
 std::mutex g_caps_mutex;
@@ -97,19 +97,11 @@ int probe_cluster(int CL) {
     return r;
 }
 
-// Cluster size for a launch of `blocks` blocks: the largest of 4 and 2 (at
-// most cmax) that divides it within the co-resident capacity, else 1.
-int cluster_for(const ClusterCaps& c, int blocks, int cmax) {
-    if (cmax >= 4 && blocks % 4 == 0 && blocks <= c.cap[2]) return 4;
-    if (cmax >= 2 && blocks % 2 == 0 && blocks <= c.cap[1]) return 2;
-    return 1;
-}
-
 int clamp_order(int P) { return P == 3 || P == 4 ? P : 2; }
 
-ClusterCaps caps_of(int dev, bool fp32, int P) {
+MmaCaps caps_of(int dev, bool fp32, int P) {
     std::lock_guard<std::mutex> lk(g_caps_mutex);
-    return (dev >= 0 && dev < kMaxDevices) ? g_dev[dev].caps[fp32][clamp_order(P)] : ClusterCaps{};
+    return dev >= 0 && dev < kMaxDevices ? g_dev[dev].mma[fp32][clamp_order(P)] : MmaCaps{};
 }
 
 bool cluster_checked(int dev) {
@@ -118,8 +110,61 @@ bool cluster_checked(int dev) {
 }
 }  // namespace
 
+namespace {
+// Shared-memory opt-in and co-resident capacity of the tensor-core kernels.
+template <typename K>
+int mma_init(K kern, int dev, int sms, bool clusters, MmaCaps& c) {
+    int optin = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    size_t room = 0;
+    for (int q = 0; q < 4; ++q) {   // the three forms, and the narrow one in clusters
+        cudaFuncAttributes fa;
+        const void* f = kern.mma_kernel(q == 3 ? 4 : 1, q == 3 ? 0 : q);
+        if (cudaFuncGetAttributes(&fa, f) != cudaSuccess) return -1;
+        const size_t dyn = (size_t)optin - fa.sharedSizeBytes;
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return -1;
+        room = room == 0 || dyn < room ? dyn : room;
+    }
+    c.bytes = room;
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern.mma_kernel(1, 2), kern.mma_threads(), room) !=
+        cudaSuccess)
+        return -1;
+    c.cap1 = per > 0 ? sms : 0;
+    c.cap4 = 0;
+    if (clusters) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[2];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 4;
+        at[0].val.clusterDim.y = 1;
+        at[0].val.clusterDim.z = 1;
+        at[1].id = cudaLaunchAttributeCooperative;
+        at[1].val.cooperative = 1;
+        cfg.gridDim = dim3(4);
+        cfg.blockDim = dim3(kern.mma_threads());
+        cfg.dynamicSmemBytes = room;
+        cfg.attrs = at;
+        cfg.numAttrs = 2;
+        int nc = 0;
+        if (cudaOccupancyMaxActiveClusters(&nc, kern.mma_kernel(4, 0), &cfg) == cudaSuccess) c.cap4 = 4 * nc;
+        else cudaGetLastError();
+    }
+    const void* f = kern.stream_kernel();
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kern.stream_bytes()) != cudaSuccess ||
+        cudaFuncSetAttribute(kern.stream_one_kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kern.stream_bytes()) != cudaSuccess)
+        return -1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, f, kern.mma_threads(), kern.stream_bytes()) != cudaSuccess ||
+        per < 1)
+        return -1;
+    c.ready = true;
+    return 0;
+}
+}  // namespace
+
 int krylov_cluster_max() {
-    // WRC_KRYLOV_CLUSTER = 1 or 2 caps the cluster size (default 4)
+    // WRC_KRYLOV_CLUSTER = 1 or 2 keeps launches unclustered (clusters are of four blocks)
     int cmax = 4;
     if (const char* ev = getenv("WRC_KRYLOV_CLUSTER")) cmax = atoi(ev) >= 4 ? 4 : (atoi(ev) >= 2 ? 2 : 1);
     return cmax;
@@ -128,12 +173,9 @@ int krylov_cluster_max() {
 int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
     if (dev < 0 || dev >= kMaxDevices) return -1;
     P = clamp_order(P);
-    int sms = 0, per = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const cudaError_t e = fp32 ? by_order<float>(P, [&](auto K) { return K.occupancy(&per); })
-                               : by_order<double>(P, [&](auto K) { return K.occupancy(&per); });
-    if (e != cudaSuccess || per < 1) return -2;
-    *max_blocks = sms * per;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return -2;
+    *max_blocks = sms;
     std::lock_guard<std::mutex> lk(g_caps_mutex);
     if (g_test_refuse < 0) {
         const char* ev = getenv("WRC_KRYLOV_TEST_REFUSE");
@@ -142,37 +184,81 @@ int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
     DeviceClusters& D = g_dev[dev];
     if (!D.probed) {
         // a launch path that does not form clusters (some profilers replay a
-        // cooperative launch without them): use the unclustered kernel
-        D.formed[1] = probe_cluster(2) == 1;
-        D.formed[2] = probe_cluster(4) == 1;
+        // cooperative launch without them): launch without
+        D.formed4 = probe_cluster(4) == 1;
         D.probed = true;
     }
-    ClusterCaps& c = D.caps[fp32][P];
+    MmaCaps& c = D.mma[fp32][P];
     if (c.ready) return 0;
-    c.cap[0] = sms * per;
-    for (int q = 1; q <= 2; ++q)
-        c.cap[q] = !D.formed[q] ? 0
-                   : fp32 ? by_order<float>(P, [&](auto K) { return K.cluster_capacity(1 << q); })
-                          : by_order<double>(P, [&](auto K) { return K.cluster_capacity(1 << q); });
-    c.ready = true;
-    return 0;
+    const int r = fp32 ? by_order<float>(P, [&](auto K) { return mma_init(K, dev, sms, D.formed4, c); })
+                       : by_order<double>(P, [&](auto K) { return mma_init(K, dev, sms, D.formed4, c); });
+    return r != 0 ? -3 : 0;
 }
 
-int krylov_step_blocks(long long n, int max_blocks, bool fp32, int P, int dev, int cmax) {
-    const ClusterCaps c = caps_of(dev, fp32, P);
-    long long b = (n + kPT - 1) / kPT;
-    if (b < 1) b = 1;
-    if (b > max_blocks) b = max_blocks;
-    // padded to a whole number of clusters where that fits (the extra blocks
-    // have no points and contribute zero partial sums)
-    const long long b4 = (b + 3) / 4 * 4, b2 = (b + 1) / 2 * 2;
-    if (cmax >= 4 && b4 <= c.cap[2] && b4 <= max_blocks) return (int)b4;
-    if (cmax >= 2 && b2 <= c.cap[1] && b2 <= max_blocks) return (int)b2;
-    return (int)b;
-}
-
-int krylov_step_cluster(long long n, int max_blocks, bool fp32, int P, int dev, int cmax) {
-    return cluster_for(caps_of(dev, fp32, P), krylov_step_blocks(n, max_blocks, fp32, P, dev, cmax), cmax);
+// Launch rule.  The kernel with its table in shared memory takes every problem
+// that fits one block per SM; beyond, the streaming one.  Points per
+// block: spread over all SMs, but at least 32 (one full warp of the operator;
+// 128^2, 2.7K points: 207 us per launch at 32, 217 at 64, 231 at 128).  The
+// narrow form up to 128 columns (points and ghosts) a block, digits as
+// halves while they fit (~370 columns at m = 30), else 64-bit integers
+// (~720): halves and integers measure the same at 220 columns (393 and 394
+// us), the integers being the only form beyond.  Clusters of four blocks,
+// which add their sums in distributed shared memory before the grid's, for
+// launches of at most 96 blocks: above, unclustered launches are faster (142
+// blocks: 317 us against 333) and use all SMs.
+// Measured on GB300, one launch, against the kernel with FP64 dots that was
+// used before: 128^2
+// pair, m = 20, 2.7K points 353 -> 207 us; m = 30: 256^2 mixed, 10.8K points
+// 559 -> 317; 1024^2, 17.0K points 483 -> 322; 4096^2 mixed, 28.8K points
+// 752 -> 393; 1024^2, 95.3K points 1321 -> 686; order 2p = 6, 7.4K points
+// 628 -> 370.
+KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int dev, int cmax) {
+    KrylovPlan K;
+    const MmaCaps c = caps_of(dev, fp32, P);
+    const auto up16 = [](long long x) { return (int)((x + 15) / 16 * 16); };
+    {
+        int ppb = up16((n + c.cap1 - 1) / std::max(1, c.cap1));
+        if (ppb < 32) ppb = 32;
+        int nb = (int)((n + ppb - 1) / ppb);
+        nb = nb < 1 ? 1 : nb;
+        int cl = 1;
+        const int b4 = (nb + 3) / 4 * 4;
+        if (cmax >= 4 && b4 <= 96 && b4 <= c.cap4) {
+            cl = 4;
+            nb = b4;
+        }
+        int gpb = up16((ng + nb - 1) / nb), form = 0;
+        const auto bytes = [&](int nrc) {
+            return fp32 ? by_order<float>(P, [&](auto kk) { return kk.mma_bytes(form, m, ppb, gpb, nrc); })
+                        : by_order<double>(P, [&](auto kk) { return kk.mma_bytes(form, m, ppb, gpb, nrc); });
+        };
+        if (ppb + gpb > 128) {
+            form = 1;
+            if (bytes(-1) > c.bytes) form = 2;
+            cl = 1;                    // clusters in the narrow form only
+        }
+        size_t need = bytes(-1);
+        if (need <= c.bytes && ppb <= 1024) {
+            K.form = form;
+            K.nrc = -1;
+            if (bytes(0) <= c.bytes) {
+                // the ghosts' interpolation rows in shared memory too, as many as fit
+                const size_t per = bytes(2) - bytes(0);
+                K.nrc = (int)((c.bytes - bytes(0)) / per * 2);
+                if (K.nrc > gpb) K.nrc = gpb;
+                need = bytes(K.nrc);
+            }
+            K.blocks = nb;
+            K.cluster = cl;
+            K.ppb = ppb;
+            K.gpb = gpb;
+            K.smem = need;
+            return K;
+        }
+    }
+    K.form = 3;
+    K.blocks = std::max(1, c.cap1);
+    return K;
 }
 
 void krylov_clusters_unformed(int dev) {
@@ -180,9 +266,9 @@ void krylov_clusters_unformed(int dev) {
     std::lock_guard<std::mutex> lk(g_caps_mutex);
     DeviceClusters& D = g_dev[dev];
     D.checked = true;
-    D.formed[1] = D.formed[2] = false;
-    for (auto& byp : D.caps)
-        for (auto& cc : byp) cc.cap[1] = cc.cap[2] = 0;
+    D.formed4 = false;
+    for (auto& byp : D.mma)
+        for (auto& cc : byp) cc.cap4 = 0;
 }
 
 // The first clustered launch on a device is checked: the stream is
@@ -193,15 +279,12 @@ void krylov_clusters_unformed(int dev) {
 // runs unclustered all the same and is seen at the step's host
 // synchronisation.
 template <typename T>
-cudaError_t launch_krylov_step(const KrylovStepArgs& args, int blocks, cudaStream_t s, int dev, int cmax) {
-    const bool fp32 = sizeof(T) == 4;
+cudaError_t launch_krylov_step(const KrylovStepArgs& args, const KrylovPlan& plan, cudaStream_t s, int dev) {
     const int P = clamp_order(args.g.P);
-    const ClusterCaps c = caps_of(dev, fp32, P);
-    const int cl = cluster_for(c, blocks, cmax);
-    const bool check = cl > 1 && !cluster_checked(dev);
+    const bool check = plan.cluster > 1 && !cluster_checked(dev);
     KrylovStepArgs a = args;
     a.refuse = (check && g_test_refuse == 1) ? 1 : 0;
-    cudaError_t e = by_order<T>(P, [&](auto K) { return K.launch(a, blocks, cl, s); });
+    cudaError_t e = by_order<T>(P, [&](auto K) { return K.launch(a, plan, s); });
     if (e != cudaSuccess) return e;
     note_launch();
     e = cudaGetLastError();
@@ -220,38 +303,82 @@ cudaError_t launch_krylov_step(const KrylovStepArgs& args, int blocks, cudaStrea
     return e;
 }
 
-template cudaError_t launch_krylov_step<double>(const KrylovStepArgs&, int, cudaStream_t, int, int);
-template cudaError_t launch_krylov_step<float>(const KrylovStepArgs&, int, cudaStream_t, int, int);
+template cudaError_t launch_krylov_step<double>(const KrylovStepArgs&, const KrylovPlan&, cudaStream_t, int);
+template cudaError_t launch_krylov_step<float>(const KrylovStepArgs&, const KrylovPlan&, cudaStream_t, int);
 
-size_t krylov_partials_doubles(int max_blocks) { return (size_t)3 * max_blocks * kOutP; }
+size_t krylov_partials_doubles() { return 2 * 8 * 128 + 16; }   // krylov_mma.cuh: sums and exponent slots
 
-int krylov_batch_max_blocks(bool fp32, int P, int pt, bool pair) {
-    int dev = 0, sms = 0, per = 0;
+int krylov_batch_max_runs(int pt) {
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const void* k = fp32 ? by_order<float>(P, [&](auto K) { return K.batch_kernel(pt, pair); })
-                         : by_order<double>(P, [&](auto K) { return K.batch_kernel(pt, pair); });
-    if (!k) return -1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, pt, 0) != cudaSuccess || per < 1) return -2;
-    return sms * per;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
+    return sms * (pt == 64 ? 8 : 4);
+}
+
+// Blocks of a batched launch, one per SM.  Up to as many problems as blocks:
+// each gets one, and the rest go one by one to the problem with the most
+// points per block, as long as its share stays above `least` points.  (A
+// launch of 48 mixed members of 9-17K points takes 4.09 ms so, 17 FP64
+// members 1.79, omega and r_v of 65.9K points 1.21; with FP64 dots, 581 and
+// 600 smaller blocks, 5.56, 2.57 and 2.06.)  More problems than blocks: whole problems, the largest first, each to
+// the block with the fewest points so far.
+void krylov_batch_plan(const std::vector<long long>& n, long long least, int sms, std::vector<int>& items,
+                       std::vector<int>& off) {
+    const int M = (int)n.size();
+    items.clear();
+    off.assign(1, 0);
+    if (M <= sms) {
+        std::vector<int> nb(M, 1);
+        for (int used = M; used < sms; ++used) {
+            int best = -1;
+            double most = (double)least;
+            for (int q = 0; q < M; ++q) {
+                const double share = (double)n[q] / nb[q];
+                if (share > most) {
+                    most = share;
+                    best = q;
+                }
+            }
+            if (best < 0) break;
+            nb[best] += 1;
+        }
+        for (int q = 0; q < M; ++q)
+            for (int b = 0; b < nb[q]; ++b) {
+                items.insert(items.end(), {q, b, nb[q]});
+                off.push_back((int)items.size() / 3);
+            }
+        return;
+    }
+    std::vector<int> order(M);
+    std::iota(order.begin(), order.end(), 0);
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
+    std::vector<std::vector<int>> bin(sms);
+    std::vector<long long> load(sms, 0);
+    for (int q : order) {
+        const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        bin[b].push_back(q);
+        load[b] += n[q];
+    }
+    for (const auto& v : bin) {
+        for (int q : v) items.insert(items.end(), {q, 0, 1});
+        off.push_back((int)items.size() / 3);
+    }
 }
 
 template <typename T>
-cudaError_t launch_krylov_batch(const KrylovStepArgs* d_args, const int* d_blk2mem, const int* d_mem_b0,
-                                int members, int blocks, int pt, int P, cudaStream_t s, bool pair) {
-    void* params[] = {(void*)&d_args, (void*)&d_blk2mem, (void*)&d_mem_b0};
-    const void* k = by_order<T>(P, [&](auto K) { return K.batch_kernel(pt, pair); });
-    if (!k) return cudaErrorInvalidValue;
-    cudaError_t e = cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(pt), params, 0, s);
+cudaError_t launch_krylov_batch(const KrylovStepArgs* d_args, const int* d_items, const int* d_off, int blocks, int P,
+                                cudaStream_t s) {
+    void* params[] = {(void*)&d_args, (void*)&d_items, (void*)&d_off};
+    const cudaError_t e = by_order<T>(P, [&](auto K) {
+        return cudaLaunchCooperativeKernel(K.stream_kernel(), dim3(blocks), dim3(K.mma_threads()), params,
+                                           K.stream_bytes(), s);
+    });
     if (e != cudaSuccess) return e;
     note_launch();
-    (void)members;
     return cudaGetLastError();
 }
 
-template cudaError_t launch_krylov_batch<double>(const KrylovStepArgs*, const int*, const int*, int, int, int, int,
-                                                 cudaStream_t, bool);
-template cudaError_t launch_krylov_batch<float>(const KrylovStepArgs*, const int*, const int*, int, int, int, int,
-                                                cudaStream_t, bool);
+template cudaError_t launch_krylov_batch<double>(const KrylovStepArgs*, const int*, const int*, int, int, cudaStream_t);
+template cudaError_t launch_krylov_batch<float>(const KrylovStepArgs*, const int*, const int*, int, int, cudaStream_t);
 
 }  // namespace wrc

@@ -1,6 +1,6 @@
 // Krylov kernels of DD order 2p = 8 (single-run and batched, FP64 and the
 // mixed mode), compiled in a translation unit of their own.
-#include "krylov_impl.cuh"
+#include "krylov_stream.cuh"
 
 namespace wrc {
 template struct KrylovKernels<double, 4>;

@@ -172,7 +172,7 @@ void pick_shape(const wrc_server* S, BatchCtx& C, const std::vector<wrc_run*>& r
             ept = tept;
         }
     }
-    if ((int)runs.size() > krylov_batch_max_blocks(C.fp32, C.P, pt)) pt = 64;
+    if ((int)runs.size() > krylov_batch_max_runs(pt)) pt = 64;
     C.pt = pt;
     C.ept = ept;
 }
@@ -238,6 +238,7 @@ void serve(wrc_server* S) {
                 if (st != WRC_OK) msg = wrc_last_error(nullptr);
             }
             if (st == WRC_OK) {
+                if (S->cfg.policy == WRC_SERVE_BATCHED) mark_batched(R);
                 st = wrc_init_vortices(R, (int32_t)q->xc.size(), q->xc.data(), q->yc.data(), q->gamma.data(),
                                        q->s.data());
                 if (st != WRC_OK) {
@@ -409,14 +410,12 @@ wrc_status wrc_server_create(const wrc_server_config* cfg, wrc_server** out) {
     if (!(cfg->hbm_budget_bytes > 0) || !std::isfinite(cfg->hbm_budget_bytes)) return bad("hbm_budget_bytes must be > 0");
     if (cfg->policy == WRC_SERVE_BATCHED) {
         // every resident run needs one block of the batched launch at least
-        for (int f = 0; f < 2 * 3; ++f) {
-            const int lim = krylov_batch_max_blocks(f >= 3, 2 + f % 3, 64);
-            if (lim <= 0) {
-                g_srv_create_error = "batched Krylov kernel occupancy query failed";
-                return WRC_ERR_CUDA;
-            }
-            if (cfg->max_slots > lim) return bad("max_slots exceeds the co-resident blocks of the batched kernel");
+        const int lim = krylov_batch_max_runs(64);
+        if (lim <= 0) {
+            g_srv_create_error = "batched Krylov kernel occupancy query failed";
+            return WRC_ERR_CUDA;
         }
+        if (cfg->max_slots > lim) return bad("max_slots exceeds the co-resident blocks of the batched kernel");
     }
     wrc_server* S = new wrc_server();
     S->cfg = *cfg;
