@@ -2178,6 +2178,7 @@ double wrc::run_bytes_for(const wrc_config& cfg, long long na, long long ng) {
     double b = 7.0 * es * N + 6.0 * N + 8.0 * N + 8.0 * nblk * kMaxKeys + 16.0 * N;
     // FFT tables: twiddles, symbols
     b += 4.0 * es * std::sqrt(N) + 16.0 * std::sqrt(N);
+    if (cfg.prec != WRC_MIXED) b += 4.0 * N + 8.0 * std::sqrt(N);   // the solve's table
     // Krylov small arrays and partial sums (at most kMaxBlocks blocks)
     b += 8.0 * (m1 * cfg.krylov_m + 33) +
          8.0 * (double)std::max(krylov_partials_doubles(), (size_t)kMaxBlocks * 4);
@@ -2197,6 +2198,7 @@ double wrc::run_device_bytes(const wrc_run* R) {
     const double nblk = std::ceil(N / kTile);
     double b = 7.0 * es * N + 6.0 * N + 8.0 * N + 8.0 * nblk * kMaxKeys + (double)R->lat64.bytes;
     b += 4.0 * es * R->g.NJ + 16.0 * R->g.NJ;
+    if (!R->fp32) b += 4.0 * N + 8.0 * R->g.NJ;
     b += 8.0 * (m1 * cfg.krylov_m + 33) +
          8.0 * (double)std::max(krylov_partials_doubles(), (size_t)kMaxBlocks * 4);
     const DevBuf* bufs[] = {&R->meta[0], &R->meta[1], &R->omega[0], &R->omega[1], &R->Ua, &R->Va, &R->ga,

@@ -14,7 +14,8 @@
 // Each FFT runs radix-16 Stockham passes (a radix-2/4/8 pass first when log2 n
 // is not a multiple of 4) on 16 values per thread held in registers, and
 // exchanges them through padded shared memory between passes (two exchanges
-// for n = 4096); no bit reversal.
+// for n = 4096); no bit reversal.  These are the FP32 ones; an FP64 run's
+// transforms are in fft_fixed.cuh.
 #include <type_traits>
 
 #include <cstdlib>
@@ -605,6 +606,8 @@ bool poison_rows() {
     return v && std::atoi(v) != 0;
 }
 
+#include "fft_fixed.cuh"
+
 template <typename T, int E, int R0>
 struct Shape {
     static int setup() {
@@ -680,8 +683,12 @@ struct Shape {
 
 template <typename T>
 int setup_all() {
-    return Shape<T, 8, 1>::setup() | Shape<T, 16, 1>::setup() | Shape<T, 16, 2>::setup() |
-           Shape<T, 16, 4>::setup() | Shape<T, 16, 8>::setup();
+    if constexpr (std::is_same<T, double>::value)
+        return FxShape<4, 1>::setup() | FxShape<4, 2>::setup() | FxShape<8, 1>::setup() | FxShape<8, 2>::setup() |
+               FxShape<8, 4>::setup();
+    else
+        return Shape<T, 8, 1>::setup() | Shape<T, 16, 1>::setup() | Shape<T, 16, 2>::setup() |
+               Shape<T, 16, 4>::setup() | Shape<T, 16, 8>::setup();
 }
 
 template <typename T>
@@ -693,10 +700,19 @@ int plan_init_t(PoissonPlan& p, const Geom& g, cudaStream_t s) {
     if (setup_all<T>() != 0) return -2;
     { launch_pdl(k_fft_init<T>, (p.n + 255) / 256, 256, 0, s, (cx_t<T>*)p.tw, (T*)p.sigma, (T*)p.dsym, p.n,
                                                        g.h, g.P); note_launch(); }
-    const int E = p.logn < 4 ? 8 : 16;
-    const int R0 = p.logn < 4 ? 1 : 1 << (p.logn % 4);
-    { k_fft_pass_tables<cx_t<T>><<<(p.n + 255) / 256, 256, 0, s>>>((const cx_t<T>*)p.tw, (cx_t<T>*)p.ptw, p.n,
-                                                                    p.logn, E, R0); note_launch(); }
+    if constexpr (std::is_same<T, double>::value) {
+        const size_t N = (size_t)(p.n / 2 + 1) * p.n;
+        if (cudaMalloc(&p.inv, sizeof(double) * N) != cudaSuccess) return -1;
+        k_fx_pass_tables<<<(p.n + 255) / 256, 256, 0, s>>>((int4*)p.ptw, p.n, p.logn, fx_log_e(p.logn));
+        k_fx_symbol<<<blocks_for((long long)N), kThreads, 0, s>>>((double*)p.inv, (const double*)p.sigma, p.n);
+        note_launch();
+    } else {
+        const int E = p.logn < 4 ? 8 : 16;
+        const int R0 = p.logn < 4 ? 1 : 1 << (p.logn % 4);
+        k_fft_pass_tables<cx_t<T>><<<(p.n + 255) / 256, 256, 0, s>>>((const cx_t<T>*)p.tw, (cx_t<T>*)p.ptw, p.n,
+                                                                      p.logn, E, R0);
+    }
+    note_launch();
     return cudaGetLastError() == cudaSuccess ? 0 : -3;
 }
 
@@ -715,6 +731,8 @@ void poisson_plan_free(PoissonPlan& p) {
     if (p.ptw) cudaFree(p.ptw);
     p.ptw = nullptr;
     if (p.sigma) cudaFree(p.sigma);
+    if (p.inv) cudaFree(p.inv);
+    p.inv = nullptr;
     if (p.dsym) cudaFree(p.dsym);
     p.tw = nullptr;
     p.sigma = nullptr;
@@ -724,17 +742,29 @@ void poisson_plan_free(PoissonPlan& p) {
 template <typename T>
 void launch_poisson(const PoissonPlan& p, const T* R, T* psi, void* C1v, void* C2v, const Geom& g, cudaStream_t s,
                     T* U, T* V, void* C3v, T* S11, T* S12, void* C4v, const int* rows) {
-    using C = cx_t<T>;
-    C* C1 = (C*)C1v;
-    C* C2 = (C*)C2v;
-    C* C3 = (C*)C3v;
-    C* C4 = (C*)C4v;
     const int logn = p.logn;
-    if (logn < 4) Shape<T, 8, 1>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
-    else if (logn % 4 == 0) Shape<T, 16, 1>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
-    else if (logn % 4 == 1) Shape<T, 16, 2>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
-    else if (logn % 4 == 2) Shape<T, 16, 4>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
-    else Shape<T, 16, 8>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
+    if constexpr (std::is_same<T, double>::value) {   // psi alone: U, V and the strain are differences of it
+        double2* C1 = (double2*)C1v;
+        if (fx_log_e(logn) == 2) {
+            if (logn % 2 == 0) FxShape<4, 1>::run(p, R, psi, C1, s, rows);
+            else FxShape<4, 2>::run(p, R, psi, C1, s, rows);
+        } else {
+            if (logn % 3 == 0) FxShape<8, 1>::run(p, R, psi, C1, s, rows);
+            else if (logn % 3 == 1) FxShape<8, 2>::run(p, R, psi, C1, s, rows);
+            else FxShape<8, 4>::run(p, R, psi, C1, s, rows);
+        }
+    } else {
+        using C = cx_t<T>;
+        C* C1 = (C*)C1v;
+        C* C2 = (C*)C2v;
+        C* C3 = (C*)C3v;
+        C* C4 = (C*)C4v;
+        if (logn < 4) Shape<T, 8, 1>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
+        else if (logn % 4 == 0) Shape<T, 16, 1>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
+        else if (logn % 4 == 1) Shape<T, 16, 2>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
+        else if (logn % 4 == 2) Shape<T, 16, 4>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
+        else Shape<T, 16, 8>::run(p, R, psi, C1, C2, s, U, V, C3, S11, S12, C4, rows);
+    }
     (void)g;
 }
 

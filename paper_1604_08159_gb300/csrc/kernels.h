@@ -68,6 +68,7 @@ struct PoissonPlan {
     void* ptw = nullptr;     // the same twiddles as per-pass tables (see fft.cu)
     void* sigma = nullptr;   // symbol of the 4th-order second-derivative stencil
     void* dsym = nullptr;    // symbol of the 4th-order first-derivative stencil (imaginary part)
+    void* inv = nullptr;     // FP64: 1/(n^2 (sigma(kx) + sigma(ky))), kx <= n/2 (see fft_fixed.cuh)
 };
 int poisson_plan_init(PoissonPlan& p, const Geom& g, bool fp32, cudaStream_t s);
 void poisson_plan_free(PoissonPlan& p);
