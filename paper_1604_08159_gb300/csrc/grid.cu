@@ -209,11 +209,13 @@ constexpr int kReconSmemMax = 160 * 1024;
 bool recon_tiles_layout(const Geom& g, size_t es, ReconTiles& lay) {
     if (g.J >= kReconLevels) return false;
     const int E = 2 * g.P - 1;
-    // tile edge: 64 up to 1024^2 (on GB300 at 1024^2, J = 5: 64 before 32, 16
-    // and the level-by-level kernels); beyond, the level-by-level kernels,
-    // whose passes then have parallelism enough (4096^2, J = 7: 0.22 ms
-    // against 0.33 ms tiled); WRC_RECON_TILE sets the edge (0: level by level)
-    int cap = g.NJ <= 1024 ? 64 : 0;
+    // tile edge: 32 up to 512^2, where larger tiles leave SMs without one, 64
+    // at 1024^2, where smaller ones recompute more (the reconstruction with
+    // its scatter, us, 64 / 32 / 16: 128^2 42 / 31 / 29, 256^2 38 / 31 / 30,
+    // 512^2 55 / 47 / 57, 1024^2 61 / 67 / 134); beyond, the level-by-level
+    // kernels, whose passes then have parallelism enough (4096^2, J = 7: 0.22
+    // ms against 0.33 ms tiled); WRC_RECON_TILE sets the edge (0: level by level)
+    int cap = g.NJ <= 512 ? 32 : g.NJ <= 1024 ? 64 : 0;
     if (const char* v = std::getenv("WRC_RECON_TILE")) cap = std::atoi(v);
     if (cap < 8) return false;   // 0: the level-by-level kernels
     for (int ts = g.NJ < cap ? g.NJ : cap; ts >= 8 && ts <= g.NJ; ts /= 2) {
@@ -553,8 +555,34 @@ __device__ __forceinline__ void for_predictor_points(int i, int k, int j, const 
     }
 }
 
+// Marks the predictor points of (i, k), except where `excl` is set: the flags
+// of a line of 2P predictors in flight together, then their marks.
+template <int P>
+__device__ __forceinline__ void mark_predictors(uint8_t* __restrict__ mask, const uint8_t* __restrict__ excl, int i,
+                                                int k, int j, const Geom& g) {
+    const int sh = g.J - j, s = 1 << sh;
+    const bool oi = (i >> sh) & 1, ok = (k >> sh) & 1, line_x = oi;   // odd in both: P lines along x
+    const int lines = oi && ok ? 2 * P : 1;
+#pragma unroll 2
+    for (int b = 0; b < lines; ++b) {
+        const int kb = lines > 1 ? (k + (2 * b + 1 - 2 * P) * s) & g.mask : k;
+        long long q[2 * P];
+        uint8_t x[2 * P];
+#pragma unroll
+        for (int t = 0; t < 2 * P; ++t) {
+            const int o = (2 * t + 1 - 2 * P) * s;
+            q[t] = line_x ? ((long long)kb << g.L) + ((i + o) & g.mask) : ((long long)((k + o) & g.mask) << g.L) + i;
+            x[t] = excl ? excl[q[t]] : 0;
+        }
+#pragma unroll
+        for (int t = 0; t < 2 * P; ++t)
+            if (!x[t]) mask[q[t]] = 1;
+    }
+}
+
 // Closure under prediction for one level (finest first): every marked level-j
 // point marks its predictor points, except where `excl` is set.
+template <int P>
 __global__ void k_closure_level(uint8_t* __restrict__ mask, const uint8_t* __restrict__ excl, int j, Geom g) {
     pdl_wait();
     const long long cnt = level_count(j, g);
@@ -562,91 +590,90 @@ __global__ void k_closure_level(uint8_t* __restrict__ mask, const uint8_t* __res
          t += (long long)gridDim.x * blockDim.x) {
         int i, k;
         level_point(t, j, g, i, k);
-        if (!mask[((long long)k << g.L) + i]) continue;
-        for_predictor_points(i, k, j, g, [&](int qi, int qk) {
-            const long long q = ((long long)qk << g.L) + qi;
-            if (!excl || !excl[q]) mask[q] = 1;
-        });
+        if (mask[((long long)k << g.L) + i]) mark_predictors<P>(mask, excl, i, k, j, g);
     }
     pdl_trigger();
 }
 
-// The closure pass of the finest level J, 16 consecutive lattice points per
+// The closure pass of the finest level J, V consecutive lattice points per
 // thread: their level-J marks (odd row or odd column) are read as separate
 // bytes, all in flight, and never the coarser points' bytes, which the pass
 // writes.
+template <int P, int V>
 __global__ void k_closure_fine(uint8_t* __restrict__ mask, const uint8_t* __restrict__ excl, Geom g) {
     pdl_wait();
-    const long long N16 = (long long)g.NJ * g.NJ / 16;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N16;
+    const long long NV = (long long)g.NJ * g.NJ / V;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < NV;
          c += (long long)gridDim.x * blockDim.x) {
-        uint8_t b[16];
+        uint8_t b[V];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const long long p = 16 * c + u;
+        for (int u = 0; u < V; ++u) {
+            const long long p = V * c + u;
             const int i = (int)(p & g.mask), k = (int)(p >> g.L);
             b[u] = ((i | k) & 1) ? mask[p] : 0;
         }
-        for (int u = 0; u < 16; ++u) {
+        for (int u = 0; u < V; ++u) {
             if (!b[u]) continue;
-            const long long p = 16 * c + u;
-            const int i = (int)(p & g.mask), k = (int)(p >> g.L);
-            for_predictor_points(i, k, g.J, g, [&](int qi, int qk) {
-                const long long q = ((long long)qk << g.L) + qi;
-                if (!excl || !excl[q]) mask[q] = 1;
-            });
+            const long long p = V * c + u;
+            mark_predictors<P>(mask, excl, (int)(p & g.mask), (int)(p >> g.L), g.J, g);
         }
     }
     pdl_trigger();
 }
 
-// Stencil levels and ghost marks (each thread reads the flags of 16
-// consecutive lattice points at once, NJ^2 being a multiple of 64, and
-// skips them when none is a grid point).  For an active point P of level l the
+// V consecutive flags (0 or 1) as bits.
+template <int V>
+__device__ __forceinline__ unsigned flag_bits(const uint8_t* __restrict__ f, long long c) {
+    static_assert(V == 1 || V == 4, "");
+    return V == 1 ? f[c] : reinterpret_cast<const unsigned*>(f)[c] * 0x01020408u >> 24 & 0xfu;
+}
+
+// Stencil levels and ghost marks (each thread reads the flags of V
+// consecutive lattice points at once, and skips those that are no grid
+// point).  For an active point P of level l the
 // stencil level along x is the largest j in [l, J] with an active point at
 // P +- h_j e_x (l if none); the stencils read P +- r h_{j*}, r = 1 .. R
 // (R = 2 for 2P = 4, max(2P - 2, P) in general), and the non-active ones
 // among them are ghosts.  Same along y.
+// Bound by the chains of dependent loads: the flags of all levels are read
+// before any is looked at.
+template <int V>
 __global__ void k_stencil_ghost(const uint8_t* __restrict__ act, uint8_t* __restrict__ gho,
                                 uint8_t* __restrict__ JJ, Geom g) {
     pdl_wait();
-    const long long N16 = (long long)g.NJ * g.NJ / 16;
+    const long long NV = (long long)g.NJ * g.NJ / V;
     const int R = dd_reach(g.P);
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N16;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < NV;
          c += (long long)gridDim.x * blockDim.x) {
-        const uint4 v = reinterpret_cast<const uint4*>(act)[c];
-        if (!(v.x | v.y | v.z | v.w)) continue;
-        const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
-        for (int u = 0; u < 16; ++u) {
-            if (!((wv[u >> 2] >> (8 * (u & 3))) & 0xffu)) continue;
-            const long long p = 16 * c + u;
+        for (unsigned bits = flag_bits<V>(act, c); bits; bits &= bits - 1) {
+            const long long p = V * c + (__ffs(bits) - 1);
             const int i = (int)(p & g.mask), k = (int)(p >> g.L);
             const int lev = level_of(i, k, g.J);
             const uint8_t* row = act + ((long long)k << g.L);
-            int jx = lev, jy = lev;
+            unsigned mx = 1u << lev, my = 1u << lev;
+#pragma unroll 4
             for (int j = g.J; j > lev; --j) {
                 const int s = 1 << (g.J - j);
-                if (row[(i + s) & g.mask] || row[(i - s) & g.mask]) {
-                    jx = j;
-                    break;
-                }
+                const unsigned x = row[(i + s) & g.mask] | row[(i - s) & g.mask];
+                const unsigned y = act[((long long)((k + s) & g.mask) << g.L) + i] |
+                                   act[((long long)((k - s) & g.mask) << g.L) + i];
+                mx |= (x ? 1u : 0u) << j;
+                my |= (y ? 1u : 0u) << j;
             }
-            for (int j = g.J; j > lev; --j) {
-                const int s = 1 << (g.J - j);
-                if (act[((long long)((k + s) & g.mask) << g.L) + i] ||
-                    act[((long long)((k - s) & g.mask) << g.L) + i]) {
-                    jy = j;
-                    break;
-                }
-            }
+            const int jx = 31 - __clz(mx), jy = 31 - __clz(my);
             JJ[p] = (uint8_t)(jx | (jy << 4));
             const int sx = 1 << (g.J - jx), sy = 1 << (g.J - jy);
-            for (int o = -R; o <= R; ++o) {
-                if (o == 0) continue;
-                const long long qx = ((long long)k << g.L) + ((i + o * sx) & g.mask);
-                if (!act[qx]) gho[qx] = 1;
-                const long long qy = ((long long)((k + o * sy) & g.mask) << g.L) + i;
-                if (!act[qy]) gho[qy] = 1;
+#pragma unroll 2
+            for (int o = 1; o <= R; ++o) {
+                const long long xl = ((long long)k << g.L) + ((i - o * sx) & g.mask);
+                const long long xh = ((long long)k << g.L) + ((i + o * sx) & g.mask);
+                const long long yl = ((long long)((k - o * sy) & g.mask) << g.L) + i;
+                const long long yh = ((long long)((k + o * sy) & g.mask) << g.L) + i;
+                const uint8_t a = act[xl], b = act[xh], d = act[yl], e = act[yh];
+                if (!a) gho[xl] = 1;
+                if (!b) gho[xh] = 1;
+                if (!d) gho[yl] = 1;
+                if (!e) gho[yh] = 1;
             }
         }
     }
@@ -1008,10 +1035,10 @@ __device__ __forceinline__ void publish_ready(int* flag, int lane) {
 // b; 4 predictors for a 1-D prediction, 16 for the tensor product), looks up
 // its grid index and, for a ghost, its row length; the rows (up to
 // kRowStage entries each) are then staged in shared memory with all loads in
-// flight, and merged in predictor order by all lanes at once -- a row's
-// entries are distinct, so each entry either adds to one existing entry or
-// is appended, new entries in row order.  The entries, their order and their
-// sums are those of merging the terms one by one.  An entry finds its place
+// flight.  The predictors that are grid points make the row's first entries,
+// all in one round; the ghosts' rows follow in predictor order, each merged
+// by all lanes at once -- a row's entries are distinct, so each entry either
+// adds to one existing entry or is appended.  An entry finds its place
 // through a per-warp hash table in shared memory (key: the active point,
 // value: its slot in the row; open addressing, linear probing), instead of
 // a scan of the row built so far.  The predictor weights are products of
@@ -1085,11 +1112,15 @@ k_ghost_rows(const int* __restrict__ list, const int* __restrict__ lat2idx, int*
             }
         }
         __syncwarp();
+        const bool bad = lane < np && (my_id < 0 || my_id >= n_tot);
+        const bool ghost_pred = lane < np && !bad && my_id >= n_act;
+        const unsigned ghosts = __ballot_sync(0xffffffffu, ghost_pred);
         // stage the predictor rows (their loads all in flight)
-        for (int q = 0; q < np; ++q) {
+        for (unsigned rest = ghosts; rest; rest &= rest - 1) {
+            const int q = __ffs(rest) - 1;
             const int id = __shfl_sync(0xffffffffu, my_id, q);
             const int rl = __shfl_sync(0xffffffffu, my_rl, q);
-            if (id >= n_act && id < n_tot && lane < rl && lane < kRowStage) {
+            if (lane < rl && lane < kRowStage) {
                 const long long r = id - n_act;
                 s_pi[wid][q][lane] = row_idx[r * rmax + lane];
                 s_pw[wid][q][lane] = row_w[r * rmax + lane];
@@ -1097,18 +1128,50 @@ k_ghost_rows(const int* __restrict__ list, const int* __restrict__ lat2idx, int*
         }
         __syncwarp();
         int len = 0;
-        bool over = false;
-        for (int q = 0; q < np; ++q) {
-            const int id = __shfl_sync(0xffffffffu, my_id, q);
-            const int rl0 = __shfl_sync(0xffffffffu, my_rl, q);
-            // weight of predictor q: a product of two DD4 weights (exact), or one
-            const double w = two_d ? c_dd4w[q & 3] * c_dd4w[q >> 2] : c_dd4w[q];
-            if (id < 0 || id >= n_tot) {                 // not a grid point: record, do not read
-                over = true;
-                continue;
+        bool over = __any_sync(0xffffffffu, bad);   // not a grid point: recorded, not read
+        // adds the lanes' terms (distinct points): to their entries, or appended
+        const auto merge = [&](bool has, int my, double mw) {
+            int pos = -1;
+            if (has)
+                for (int h = row_hash(my);; h = (h + 1) & (kRowHash - 1)) {
+                    const int key = hkey[h];
+                    if (key == my) {
+                        pos = hval[h];
+                        break;
+                    }
+                    if (key < 0) break;
+                }
+            if (pos >= 0) wt[pos] += mw;
+            const unsigned fresh = __ballot_sync(0xffffffffu, has && pos < 0);
+            if (has && pos < 0) {
+                const int slot = len + __popc(fresh & ((1u << lane) - 1u));
+                if (slot < cap) {
+                    idx[slot] = my;
+                    wt[slot] = mw;
+                    // distinct keys in one round: a claimed slot is another key's
+                    for (int h = row_hash(my);; h = (h + 1) & (kRowHash - 1))
+                        if (atomicCAS(&hkey[h], -1, my) == -1) {
+                            hval[h] = slot;
+                            hpos[slot] = h;
+                            break;
+                        }
+                }
             }
-            const bool ghost = id >= n_act;
-            const int rl = ghost ? rl0 : 1;
+            const int nf = __popc(fresh);
+            if (len + nf > cap) over = true;
+            len = len + nf < cap ? len + nf : cap;
+            __syncwarp();
+        };
+        // weight of predictor q: a product of two DD4 weights (exact), or one
+        const double w_q = lane < np ? (two_d ? c_dd4w[lane & 3] * c_dd4w[lane >> 2] : c_dd4w[lane]) : 0.0;
+        // the grid points among the predictors in one round (distinct points:
+        // a level-0 lattice of at least four points a side), then the ghosts' rows
+        merge(lane < np && !bad && !ghost_pred, my_id, w_q);
+        for (unsigned rest = ghosts; rest; rest &= rest - 1) {
+            const int q = __ffs(rest) - 1;
+            const int id = __shfl_sync(0xffffffffu, my_id, q);
+            const int rl = __shfl_sync(0xffffffffu, my_rl, q);
+            const double w = __shfl_sync(0xffffffffu, w_q, q);
             const long long r = id - n_act;
             for (int e0 = 0; e0 < rl; e0 += 32) {
                 const int e = e0 + lane;
@@ -1116,10 +1179,7 @@ k_ghost_rows(const int* __restrict__ list, const int* __restrict__ lat2idx, int*
                 int my = 0;
                 double mw = 0.0;
                 if (has) {
-                    if (!ghost) {
-                        my = id;
-                        mw = w;
-                    } else if (e < kRowStage) {
+                    if (e < kRowStage) {
                         my = s_pi[wid][q][e];
                         mw = w * s_pw[wid][q][e];
                     } else {
@@ -1127,36 +1187,7 @@ k_ghost_rows(const int* __restrict__ list, const int* __restrict__ lat2idx, int*
                         mw = w * row_w[r * rmax + e];
                     }
                 }
-                int pos = -1;
-                if (has)
-                    for (int h = row_hash(my);; h = (h + 1) & (kRowHash - 1)) {
-                        const int key = hkey[h];
-                        if (key == my) {
-                            pos = hval[h];
-                            break;
-                        }
-                        if (key < 0) break;
-                    }
-                if (pos >= 0) wt[pos] += mw;
-                const unsigned fresh = __ballot_sync(0xffffffffu, has && pos < 0);
-                if (has && pos < 0) {
-                    const int slot = len + __popc(fresh & ((1u << lane) - 1u));
-                    if (slot < cap) {
-                        idx[slot] = my;
-                        wt[slot] = mw;
-                        // distinct keys in one round: a claimed slot is another key's
-                        for (int h = row_hash(my);; h = (h + 1) & (kRowHash - 1))
-                            if (atomicCAS(&hkey[h], -1, my) == -1) {
-                                hval[h] = slot;
-                                hpos[slot] = h;
-                                break;
-                            }
-                    }
-                }
-                const int nf = __popc(fresh);
-                if (len + nf > cap) over = true;
-                len = len + nf < cap ? len + nf : cap;
-                __syncwarp();
+                merge(has, my, mw);
             }
         }
         for (int e = lane; e < len; e += 32) {
@@ -1326,6 +1357,23 @@ k_ghost_rows_wide(const int* __restrict__ list, const int* __restrict__ lat2idx,
     pdl_trigger();
 }
 
+// f(half the DD order), as a constant.
+template <typename F>
+void by_order(const Geom& g, F&& f) {
+    if (g.P == 3) f(std::integral_constant<int, 3>{});
+    else if (g.P == 4) f(std::integral_constant<int, 4>{});
+    else f(std::integral_constant<int, 2>{});
+}
+// f(lattice flags per thread) for the passes over the lattice's flags, bound
+// by a thread's chain of dependent loads: one while that leaves each SM a few
+// warps, else four (the adaptation, us, one / four / sixteen: 128^2 78 / 80 /
+// 99, 256^2 79 / 83 / 105, 1024^2 103 / 99 / 104, 4096^2 264 / 201 / 202).
+template <typename F>
+void flags_per_thread(const Geom& g, F&& f) {
+    if (g.NJ <= 256) f(std::integral_constant<int, 1>{});
+    else f(std::integral_constant<int, 4>{});
+}
+
 // The ghost-row kernel of the DD order of g.
 using RowsKernel = void (*)(const int*, const int*, int*, int*, double*, int, Geom, int*, const int*, int, int*, int*,
                             unsigned long long, int);
@@ -1394,13 +1442,24 @@ void launch_details_adj(const uint32_t* meta, long long n, const T* L, double ep
 }
 void launch_closure_level(uint8_t* mask, const uint8_t* excl, int j, const Geom& g, cudaStream_t s) {
     if (j == g.J)
-        launch_pdl(k_closure_fine, blocks_for((long long)g.NJ * g.NJ / 16), kThreads, 0, s, mask, excl, g);
+        flags_per_thread(g, [&](auto v) {
+            constexpr int V = decltype(v)::value;
+            by_order(g, [&](auto p) {
+                launch_pdl(k_closure_fine<decltype(p)::value, V>, blocks_for((long long)g.NJ * g.NJ / V), kThreads, 0, s, mask, excl, g);
+            });
+        });
     else
-        launch_pdl(k_closure_level, blocks_for(level_count(j, g)), kThreads, 0, s, mask, excl, j, g);
+        by_order(g, [&](auto p) {
+            launch_pdl(k_closure_level<decltype(p)::value>, blocks_for(level_count(j, g)), kThreads, 0, s, mask, excl, j, g);
+        });
     note_launch();
 }
 void launch_stencil_ghost(const uint8_t* act, uint8_t* gho, uint8_t* JJ, const Geom& g, cudaStream_t s) {
-    { launch_pdl(k_stencil_ghost, blocks_for((long long)g.NJ * g.NJ / 16), kThreads, 0, s, act, gho, JJ, g); note_launch(); }
+    flags_per_thread(g, [&](auto v) {
+        constexpr int V = decltype(v)::value;
+        launch_pdl(k_stencil_ghost<V>, blocks_for((long long)g.NJ * g.NJ / V), kThreads, 0, s, act, gho, JJ, g);
+    });
+    note_launch();
 }
 void launch_validate_grid(const uint8_t* act, int* flag, const Geom& g, cudaStream_t s) {
     { launch_pdl(k_validate_grid, blocks_for((long long)g.NJ * g.NJ), kThreads, 0, s, act, flag, g); note_launch(); }
