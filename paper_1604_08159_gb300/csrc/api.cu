@@ -1014,6 +1014,35 @@ wrc_status exner_krylov(wrc_run* R) {
     CK(cudaMemsetAsync(R->K.H, 0, sizeof(double) * (m + 1) * m, s));
     CK(ex_scatter_fields(a, fs, Lb, nullptr, 0, s));
     CK(ex_base(a, K.w, s));
+    const KrylovPlan plan = krylov_ex_plan(n, R->n_ghost, m, R->g.P, R->device);
+    if (plan.form < 3) {
+        KrylovStepArgs A{};
+        A.g = R->g;
+        A.meta = a.meta;
+        A.n = (int)(3 * n);
+        A.glist = a.glist;
+        A.ng = 3 * a.ng;
+        A.row_len = a.row_len;
+        A.row_idx = a.row_idx;
+        A.row_w = a.row_w;
+        A.rmax = a.rmax;
+        A.row_overflow = R->K.overflow;
+        A.w = K.w;
+        A.H = K.H;
+        A.y = K.y;
+        A.beta = K.beta;
+        A.kstop = K.kstop;
+        A.flags = K.flags;
+        A.part = K.part;
+        A.bar = K.bar;
+        A.err = K.err;
+        A.m = m;
+        A.dt = K.dt;
+        A.tol = K.tol;
+        A.limit_ns = K.limit_ns;
+        CK(launch_krylov_ex(A, a, plan, s));
+        return WRC_OK;
+    }
     CK(ex_krylov(a, K, blocks, s));
     return WRC_OK;
 }

@@ -8,7 +8,9 @@
 // stacked vector [u; v; pi] of the active points in one persistent
 // cooperative kernel: per Krylov vector its three lattices (values at the
 // active points, the ghosts through the interpolation rows), the operator
-// and classical Gram-Schmidt twice.  No Poisson solve.
+// and classical Gram-Schmidt twice -- krylov_mma.cuh's while its table fits
+// the SMs' shared memory, else k_ex_krylov here.  No Poisson solve.
+#include "exner_op.cuh"
 #include "krylov_impl.cuh"
 #include "wrc.h"
 
@@ -104,53 +106,6 @@ __global__ void k_ex_base(ExArgs a, double* __restrict__ w) {
         w[n + i] = -(u * vx + v * vy) - a.C * py - a.fc * (u - a.gx) - a.r * v + a.nu * lv;
         w[2 * n + i] = -(u * px + v * py) - p * (ux + vy);
     }
-}
-
-// M q at the active points: the frozen-coefficient operator (advection by
-// the state's velocity, pressure gradient, pi times the divergence,
-// Coriolis, friction, viscosity) plus, for the exact Jacobian, the terms of
-// the state's gradients.
-// Entry e of M q (e = f n + i: field f at active point i; M the exact
-// Jacobian with full, else the frozen-coefficient operator): the own field's
-// collocation derivatives at the point's stencil levels and the cross terms
-// of the other fields (the lattices a.Lq hold q with its ghost values).
-template <int P>
-__device__ __forceinline__ double ex_entry(const ExArgs& a, const double* __restrict__ q, int f, int i) {
-    const int n = a.n;
-    const long long ld = a.ld;
-    const uint32_t mw = a.meta[i];
-    const double* d = a.d;
-    const double u = a.f[0][i], v = a.f[1][i];
-    const double du = q[i], dv = q[n + i];
-    if (f == 0) {
-        double dx, dy, lap;
-        point_derivs<double, P>(a.Lq[0], mw, a.g, a.c1J, a.c2J, dx, dy, lap);
-        const double dpx = point_d1<double, P>(a.Lq[2], mw, a.g, a.c1J, 0);
-        double J = -(u * dx + v * dy) - a.C * dpx + a.fc * dv - a.r * du + a.nu * lap;
-        if (a.full) J -= du * d[i] + dv * d[ld + i];
-        return J;
-    }
-    if (f == 1) {
-        double dx, dy, lap;
-        point_derivs<double, P>(a.Lq[1], mw, a.g, a.c1J, a.c2J, dx, dy, lap);
-        const double dpy = point_d1<double, P>(a.Lq[2], mw, a.g, a.c1J, 1);
-        double J = -(u * dx + v * dy) - a.C * dpy - a.fc * du - a.r * dv + a.nu * lap;
-        if (a.full) J -= du * d[2 * ld + i] + dv * d[3 * ld + i];
-        return J;
-    }
-    const double dpx = point_d1<double, P>(a.Lq[2], mw, a.g, a.c1J, 0);
-    const double dpy = point_d1<double, P>(a.Lq[2], mw, a.g, a.c1J, 1);
-    const double dux = point_d1<double, P>(a.Lq[0], mw, a.g, a.c1J, 0);
-    const double dvy = point_d1<double, P>(a.Lq[1], mw, a.g, a.c1J, 1);
-    double J = -(u * dpx + v * dpy) - a.f[2][i] * (dux + dvy);
-    if (a.full) J -= (du * d[4 * ld + i] + dv * d[5 * ld + i]) + q[2 * n + i] * (d[i] + d[3 * ld + i]);
-    return J;
-}
-
-// Field and point of a stacked entry.
-__device__ __forceinline__ void ex_split(long long e, int n, int& f, int& i) {
-    f = e >= 2LL * n ? 2 : (e >= n ? 1 : 0);
-    i = (int)(e - (long long)f * n);
 }
 
 // Basis vector q_c = w * scale at the block's own stacked entries, their
@@ -345,7 +300,6 @@ __global__ void __launch_bounds__(kExKrylovThreads, 1) k_ex_krylov(ExArgs a, ExK
         ex_new_vector(a, K, 0, 1.0 / beta, e0, stride, s_dot[wid]);
         if (!grid_sync(K.bar, K.err, K.limit_ns, bid, nb)) return;
         for (int j = 0; j < m; ++j) {
-            const double* qj = K.basis + (size_t)j * K.ld3;
             const int nv = j + 1, L = ex_lanes_per_row(nv);
             // w = M q_j; c = Q^T w and |w|^2
             nrm = 0.0;
@@ -356,7 +310,7 @@ __global__ void __launch_bounds__(kExKrylovThreads, 1) k_ex_krylov(ExArgs a, ExK
                 if (e < N3) {
                     int f, i;
                     ex_split(e, n, f, i);
-                    x = ex_entry<P>(a, qj, f, i);
+                    x = ex_entry<P>(a, a.meta[i], f, i);
                     w[e] = x;
                     nrm += x * x;
                 }

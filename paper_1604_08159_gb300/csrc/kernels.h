@@ -196,7 +196,8 @@ cudaError_t ex_scatter_fields(const ExArgs& a, const double* const src[3], doubl
 cudaError_t ex_base(const ExArgs& a, double* w, cudaStream_t s);
 // Fill a lattice with a constant.
 cudaError_t ex_fill(double* F, long long n, double value, cudaStream_t s);
-// The whole Krylov projection of a velocity-Exner step in one persistent
+// The whole Krylov projection of a velocity-Exner step too large for
+// launch_krylov_ex's plans, in one persistent
 // cooperative launch (b = F(U^n) in w on entry): classical Gram-Schmidt
 // twice on the stacked vectors, four grid barriers per Arnoldi step (bounded
 // waits: bit 1 of *err on expiry), phi_1 by block 0, the update.
@@ -293,6 +294,11 @@ KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int d
 template <typename T>
 cudaError_t launch_krylov_step(const KrylovStepArgs& args, const KrylovPlan& plan, cudaStream_t s, int dev);
 size_t krylov_partials_doubles();
+// The velocity-Exner step by the same kernel over the 3 n entries of the
+// stacked vectors: its plan (form 3: they do not fit; ex_krylov then), and
+// the launch (args.w holds b = F(U^n), args.n and args.ng count entries).
+KrylovPlan krylov_ex_plan(long long n, long long ng, int m, int P, int dev);
+cudaError_t launch_krylov_ex(const KrylovStepArgs& args, const ExArgs& x, const KrylovPlan& plan, cudaStream_t s);
 // Batched Krylov step of several problems (device array of arguments) in one
 // cooperative launch of the streaming form: block b works on the items
 // d_off[b] .. d_off[b + 1] - 1, each (problem, block index in it, its
@@ -312,6 +318,7 @@ cudaError_t launch_krylov_batch(const KrylovStepArgs* d_args, const int* d_items
 template <typename T, int P>
 struct KrylovKernels {
     const void* mma_kernel(int cl, int form);
+    const void* ex_kernel(int form);   // the velocity-Exner step (FP64; null otherwise)
     int mma_threads();
     size_t mma_bytes(int form, int m, int ppb, int gpb, int nrc);
     const void* stream_kernel();

@@ -117,9 +117,10 @@ int mma_init(K kern, int dev, int sms, bool clusters, MmaCaps& c) {
     int optin = 0;
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     size_t room = 0;
-    for (int q = 0; q < 4; ++q) {   // the three forms, and the narrow one in clusters
+    for (int q = 0; q < 7; ++q) {   // the three forms, the narrow one in clusters, the velocity-Exner ones
         cudaFuncAttributes fa;
-        const void* f = kern.mma_kernel(q == 3 ? 4 : 1, q == 3 ? 0 : q);
+        const void* f = q < 4 ? kern.mma_kernel(q == 3 ? 4 : 1, q == 3 ? 0 : q) : kern.ex_kernel(q - 4);
+        if (!f) continue;
         if (cudaFuncGetAttributes(&fa, f) != cudaSuccess) return -1;
         const size_t dyn = (size_t)optin - fa.sharedSizeBytes;
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess) return -1;
@@ -259,6 +260,28 @@ KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int d
     K.form = 3;
     K.blocks = std::max(1, c.cap1);
     return K;
+}
+
+// The velocity-Exner step takes the same kernel while its 3 n entries fit
+// (up to ~30K points at m = 30): with two barriers per Arnoldi step instead of
+// the four and FP64 dots of k_ex_krylov, which runs what does not fit, a step
+// of 7.5K points at 1024^2, m = 30, takes 489 us instead of 1327.
+KrylovPlan krylov_ex_plan(long long n, long long ng, int m, int P, int dev) {
+    return krylov_plan(3 * n, 3 * ng, m, false, P, dev, 1);
+}
+
+cudaError_t launch_krylov_ex(const KrylovStepArgs& args, const ExArgs& x, const KrylovPlan& plan, cudaStream_t s) {
+    KrylovStepArgs a = args;
+    ExArgs xa = x;
+    int ppb = plan.ppb, gpb = plan.gpb, nrc = plan.nrc;
+    void* params[] = {&a, &xa, &ppb, &gpb, &nrc};
+    const cudaError_t e = by_order<double>(clamp_order(args.g.P), [&](auto K) {
+        return cudaLaunchCooperativeKernel(K.ex_kernel(plan.form), dim3(plan.blocks), dim3(K.mma_threads()), params,
+                                           plan.smem, s);
+    });
+    if (e != cudaSuccess) return e;
+    note_launch();
+    return cudaGetLastError();
 }
 
 void krylov_clusters_unformed(int dev) {

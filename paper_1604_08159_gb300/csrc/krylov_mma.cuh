@@ -37,6 +37,7 @@
 // (h, qz) while the products of the updates run.
 //
 // Measured on GB300: see krylov_plan() in krylov.cu.
+#include "exner_op.cuh"
 #include "krylov_impl.cuh"
 
 namespace wrc {
@@ -781,9 +782,13 @@ __device__ __forceinline__ void split2(double x, float& h, float& l) {
 // formed clusters of CL blocks, whose sums are added in distributed shared
 // memory first.  Returns the number of steps whose dots were taken, for
 // the cluster barriers at the end.
-template <typename T, int CL, int P, int FORM>
+// EX: the velocity-Exner step.  The points are the 3 X->n entries of the
+// stacked vector (A.n of them, field after field), the ghosts likewise, each
+// field on its own lattice; b = F(U^n) is in A.w on entry.
+template <typename T, int CL, int P, int FORM, bool EX = false>
 __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const int bid, const int nb, const int ppb,
-                                               const int gpb, const int nrc, const bool formed, char* sm) {
+                                               const int gpb, const int nrc, const bool formed, char* sm,
+                                               const ExArgs* X = nullptr) {
     constexpr bool wide = FORM != kNarrow, HALF = FORM != kWords;
     constexpr int NU = wide ? 4 : 2, cstep = 8 * NU;   // columns a product warp takes in a turn
     __shared__ double s_v[2][32];        // s (and |u|^2), t (and u.z) of a step
@@ -825,6 +830,16 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
     T* Lq = (T*)A.Lq;
     T* zb = (T*)A.w;                   // z at every active point (read by the ghosts' rows)
     const T nu = (T)A.nu, r = (T)A.r, c1J = (T)A.c1J, c2J = (T)A.c2J;
+    // field and point of stacked entry e, field and ghost of stacked ghost t; a field's lattice
+    const int xn = EX ? X->n : 0, xg = EX ? X->ng : 0;
+    const auto field = [&](long long e) { return EX ? (e >= 2LL * xn ? 2 : (e >= xn ? 1 : 0)) : 0; };
+    const auto gfield = [&](long long t) { return EX ? (t >= 2LL * xg ? 2 : (t >= xg ? 1 : 0)) : 0; };
+    const auto row_of = [&](long long t) { return EX ? t - (long long)gfield(t) * xg : t; };
+    const auto z_of = [&](long long t) { return EX ? zb + (size_t)gfield(t) * xn : zb; };
+    const auto lattice = [&](int f) {
+        if constexpr (EX) return (T*)(f == 2 ? X->Lq[2] : (f == 1 ? X->Lq[1] : X->Lq[0]));
+        else return Lq;
+    };
     // global scratch: sums [2][kCopies][64][2] (block b adds to copy b mod kCopies: with one
     // copy the additions of 152 blocks to the same words took up to 2 us), then per step
     // parity the exponents of u and of z not finite, and |A|'s
@@ -863,13 +878,14 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
         for (int c = threadIdx.x; c < (m + 1) * pitch * 4; c += kMT) reinterpret_cast<unsigned*>(Q)[c] = 0u;
     else
         for (int c = threadIdx.x; c < (m + 1) * pitch; c += kMT) reinterpret_cast<unsigned long long*>(Q)[c] = kBias;
-    for (int c = threadIdx.x; c < n; c += kMT) meta[c] = A.meta[p0 + c];
+    for (int c = threadIdx.x; c < n; c += kMT) meta[c] = A.meta[p0 + c - (EX ? (long long)field(p0 + c) * xn : 0)];
     for (int e = threadIdx.x; e < min(nrc, ng) * kRowCache; e += kMT) {
         const int q = e / kRowCache, i = e - q * kRowCache;
-        const int rl = A.row_len[t0 + q];
+        const long long t = row_of(t0 + q);
+        const int rl = A.row_len[t];
         if (i < rl && rl <= kRowCache) {
-            ri[e] = A.row_idx[(size_t)(t0 + q) * A.rmax + i];
-            rw[e] = A.row_w[(size_t)(t0 + q) * A.rmax + i];
+            ri[e] = A.row_idx[(size_t)t * A.rmax + i];
+            rw[e] = A.row_w[(size_t)t * A.rmax + i];
         }
     }
     if (threadIdx.x < 8) s_e[threadIdx.x] = 0;
@@ -883,6 +899,13 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
         int ea = 0;
         if (p < n) {
             const uint32_t mw = meta[p];
+            if constexpr (EX) {
+                const int f = field(p0 + p);
+                const T v = zb[p0 + p];
+                us[p] = dbl(v);
+                lattice(f)[meta_pos(mw)] = v;
+                ea = expo(ex_row_bound<P>(*X, mw, f, (int)(p0 + p - (long long)f * xn)));
+            } else {
             const T U = Ua[p], V = Va[p];
             T v = apply_point<T, false, P>((const T*)A.L, mw, U, V, nu, r, A.g, c1J, c2J);
             if (A.ga) v += ((const T*)A.ga)[p0 + p];
@@ -890,6 +913,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
             zb[p0 + p] = v;
             Lq[meta_pos(mw)] = v;
             ea = expo(row_bound<T, P>(A, mw, U, V));
+            }
         }
         ea = (int)__reduce_max_sync(0xffffffffu, (unsigned)ea);
         if (lane == 0) atomicMax(&s_e[6], ea);
@@ -900,16 +924,17 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
     for (int q = wid * 4; q < ng; q += 4 * kMW) {
         const int gi = q + (lane >> 3), gl = lane & 7;
         const bool valid = gi < ng;
-        const int rl = valid ? A.row_len[t0 + gi] : 0;
-        const double v = ghost_row<T>(A, zb, t0 + gi, rl, gl, nullptr, nullptr);
-        const int gs = ghost_scale(A, t0 + gi, rl, gl);
+        const long long t = row_of(t0 + gi);
+        const int rl = valid ? A.row_len[t] : 0;
+        const double v = ghost_row<T>(A, z_of(t0 + gi), t, rl, gl, nullptr, nullptr);
+        const int gs = ghost_scale(A, t, rl, gl);
         if (valid && gl == 0) {
             const T gv = (T)v;
-            const int pos = A.glist[t0 + gi];
-            gpos[gi] = pos | (gs << 24);
+            const int pos = A.glist[t], f = gfield(t0 + gi);
+            gpos[gi] = pos | (gs << 24) | (f << 29);
             glen[gi] = rl;
             us[ppb + gi] = dbl(gv);
-            Lq[pos] = gv;
+            lattice(f)[pos] = gv;
         }
     }
     __syncthreads();
@@ -935,7 +960,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
     const int opw = wid < 8 ? wid : wid - 1;             // warp 8 takes no points
     OpPoint<T> op0;
     op_prepare<T, P>(op0, 0, T(0), T(0), T(0), A.g, c1J, c2J);
-    if (wid != 8 && opw * 32 + lane < n)
+    if (!EX && wid != 8 && opw * 32 + lane < n)
         op_prepare<T, P>(op0, meta[opw * 32 + lane], Ua[opw * 32 + lane], Va[opw * 32 + lane], nu, A.g, c1J, c2J);
     const int gw = wid >= 9 ? wid - 9 : wid - 2 + 3;     // first ghost pass of this warp
     int k = m;
@@ -1005,7 +1030,10 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                 int e = 0;
                 if (p < n) {
                     T z;
-                    if (c == opw * 32) {
+                    if constexpr (EX) {
+                        const int f = field(p0 + p);
+                        z = (T)ex_entry<P>(*X, meta[p], f, (int)(p0 + p - (long long)f * xn));
+                    } else if (c == opw * 32) {
                         z = op_apply<T, P>(Lq, op0, r, A.g, c1J, c2J);
                     } else {
                         OpPoint<T> op;
@@ -1176,7 +1204,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
             // passes of four ghosts over warps 9-11, then 2-7 (which would otherwise wait for the sums)
             for (int x = gw; 4 * x < ng; x += 9) {
                 const int gi = 4 * x + (lane >> 3);
-                const double v = ghost_row<T>(A, zb, t0 + gi, gi < ng ? glen[gi] : 0, lane & 7, rw + gi * kRowCache,
+                const double v = ghost_row<T>(A, z_of(t0 + gi), row_of(t0 + gi), gi < ng ? glen[gi] : 0, lane & 7, rw + gi * kRowCache,
                                               gi < nrc ? ri + gi * kRowCache : nullptr);
                 if (gi < ng && (lane & 7) == 0) rz[gi] = v;
             }
@@ -1265,7 +1293,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                         }
                     } else if (c < Y.cols) {   // (the last turn may read past the end of the rows)
                         // in place: FP64 and the ghosts, the differences; mixed points, FP32 pairs (u, ps), (z, pc)
-                        const int gs = c >= ppb && c - ppb < ng ? gpos[c - ppb] >> 24 : 0;
+                        const int gs = c >= ppb && c - ppb < ng ? (gpos[c - ppb] >> 24) & 31 : 0;
                         if (sizeof(T) == 4 && c < ppb) {
                             if (pass == 0) {
                                 const float z = d2f_same(zs[c]), u = d2f_same(us[c]);
@@ -1323,15 +1351,15 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                         const longlong2 v = wide ? make_longlong2(0, 0) : vv[c];
                         double q1, u1;
                         const double z = gh ? (wide ? rz[c - ppb] + zs[c] : rz[c - ppb]) : zs[c];
-                        next_values(us[c], z, v.y, es - 60 + (gp >> 24), v.x, et - 60 + (gp >> 24), S, q1, u1);
+                        next_values(us[c], z, v.y, es - 60 + ((gp >> 24) & 31), v.x, et - 60 + ((gp >> 24) & 31), S, q1, u1);
                         qj = (T)q1;
                         if (sizeof(T) == 4) u1 = fma(q1 - dbl(qj), S.qz * S.hinv, u1);   // with the rounded q_j
                         un = (T)u1;
                     }
                     us[c] = dbl(un);
-                    Lq[gh ? gp & 0xffffff : meta_pos(meta[c])] = un;
+                    lattice(gh ? (gp >> 29) & 3 : field(p0 + c))[gh ? gp & 0xffffff : meta_pos(meta[c])] = un;
                     e = expo(un);
-                    put_value<HALF>(Q, pitch, dstride, j, c, fix62(qj, 1023 + (gp >> 24)));
+                    put_value<HALF>(Q, pitch, dstride, j, c, fix62(qj, 1023 + ((gp >> 24) & 31)));
                 }
                 const int ea = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
                 const int ep = (int)__reduce_max_sync(0xffffffffu, (unsigned)(gh ? 0 : e));
@@ -1383,9 +1411,17 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
             const int c = c0 + lane;
             const longlong2 v = update_sums<NU, HALF>(Q, pitch, dstride, k, c0, tile, (float*)scr);
             if (lane < cstep && c < n) {
-                const T x = (T)fma((double)v.x, sc, dbl(om[c]));
-                om[c] = x;
-                Lo[meta_pos(meta[c])] = x;
+                if constexpr (EX) {
+                    const int f = field(p0 + c), i = (int)(p0 + c - (long long)f * xn);
+                    double* F = f == 2 ? X->f_out[2] : (f == 1 ? X->f_out[1] : X->f_out[0]);
+                    const double x = fma((double)v.x, sc, F[i]);
+                    F[i] = x;
+                    (f == 2 ? X->Lb[2] : (f == 1 ? X->Lb[1] : X->Lb[0]))[meta_pos(meta[c])] = x;
+                } else {
+                    const T x = (T)fma((double)v.x, sc, dbl(om[c]));
+                    om[c] = x;
+                    Lo[meta_pos(meta[c])] = x;
+                }
             }
         }
     }
@@ -1412,8 +1448,23 @@ __global__ void __launch_bounds__(kMT, 1) k_krylov_mma(KrylovStepArgs A, int ppb
     (void)calls;
 }
 
+template <int P, int FORM>
+__global__ void __launch_bounds__(kMT, 1) k_ex_mma(KrylovStepArgs A, const __grid_constant__ ExArgs X, int ppb, int gpb,
+                                                   int nrc) {
+    extern __shared__ __align__(16) char k_sm[];
+    krylov_mma_body<double, 1, P, FORM, true>(A, blockIdx.x, gridDim.x, ppb, gpb, nrc, false, k_sm, &X);
+}
+
 }  // namespace
 
+template <typename T, int P>
+const void* KrylovKernels<T, P>::ex_kernel(int form) {
+    if constexpr (sizeof(T) == 8)
+        return form == kNarrow ? (const void*)k_ex_mma<P, kNarrow>
+                               : form == kHalves ? (const void*)k_ex_mma<P, kHalves> : (const void*)k_ex_mma<P, kWords>;
+    else
+        return nullptr;
+}
 template <typename T, int P>
 const void* KrylovKernels<T, P>::mma_kernel(int cl, int form) {
     if (form == kNarrow) return cl == 4 ? (const void*)k_krylov_mma<T, 4, P, kNarrow> : (const void*)k_krylov_mma<T, 1, P, kNarrow>;
