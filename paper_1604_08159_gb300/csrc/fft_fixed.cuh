@@ -273,16 +273,19 @@ __global__ void k_fx_symbol(double* __restrict__ inv, const double* __restrict__
     pdl_trigger();
 }
 
-// Step 1 (see k_px_fwd).
+// Step 1 (see k_px_fwd).  In these kernels the wait for the predecessor comes
+// before anything else and its data is read by coherent loads: read-only
+// loads (of const __restrict__ pointers) may be moved above a wait that
+// follows other code, where they read what the predecessor has yet to write.
 template <int E, int R0>
 __global__ void __launch_bounds__(kFxThreads) k_px_fwd_fx(const double* __restrict__ Rf, double2* __restrict__ S, int n,
                                                    int logn, const int4* __restrict__ tw) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned s_slot[kFxEvents];
     const int nt = n / E, F = blockDim.x / nt;
     const int f = threadIdx.x / nt, i = threadIdx.x - f * nt;
     FxShare sh = fx_share(s_slot, nt);
-    pdl_wait();
     const int h = n / 2;
     const int q = blockIdx.x * F + f;
     const bool on = q < h;
@@ -296,7 +299,7 @@ __global__ void __launch_bounds__(kFxThreads) k_px_fwd_fx(const double* __restri
 #pragma unroll
         for (int e = 0; e < E; ++e) {
             const int x = i + e * nt;
-            d[e] = on ? make_double2(r0[x], r1[x]) : make_double2(0.0, 0.0);
+            d[e] = on ? make_double2(__ldcg(r0 + x), __ldcg(r1 + x)) : make_double2(0.0, 0.0);
         }
         fx_from(d, v, ex, sh);
     }
@@ -329,12 +332,12 @@ __global__ void __launch_bounds__(kFxThreads) k_px_fwd_fx(const double* __restri
 template <int E, int R0>
 __global__ void __launch_bounds__(kFxThreads) k_py_solve_fx(double2* __restrict__ ST, int n, int logn,
                                                      const int4* __restrict__ tw, const double* __restrict__ inv) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned s_slot[kFxEvents];
     const int nt = n / E, F = blockDim.x / nt;
     const int f = threadIdx.x / nt, i = threadIdx.x - f * nt;
     FxShare sh = fx_share(s_slot, nt);
-    pdl_wait();
     const int h = n / 2;
     const int kx = blockIdx.x * F + f;
     const bool on = kx < h;
@@ -389,12 +392,12 @@ template <int E, int R0>
 __global__ void __launch_bounds__(kFxThreads) k_px_inv_fx(const double2* __restrict__ S, double* __restrict__ out, int n,
                                                    int logn, const int4* __restrict__ tw,
                                                    const int* __restrict__ rows) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned s_slot[kFxEvents];
     const int nt = n / E, F = blockDim.x / nt;
     const int f = threadIdx.x / nt, i = threadIdx.x - f * nt;
     FxShare sh = fx_share(s_slot, nt);
-    pdl_wait();
     const int h = n / 2;
     int q = blockIdx.x * F + f;
     if (rows) {
@@ -418,17 +421,17 @@ __global__ void __launch_bounds__(kFxThreads) k_px_inv_fx(const double2* __restr
             const int x = i + e * nt;
             double2 a, b;
             if (x == 0) {
-                a = make_double2(sa[0].x, 0.0);
-                b = make_double2(sb[0].x, 0.0);
+                a = make_double2(__ldcg(sa).x, 0.0);
+                b = make_double2(__ldcg(sb).x, 0.0);
             } else if (x == h) {
-                a = make_double2(sa[0].y, 0.0);
-                b = make_double2(sb[0].y, 0.0);
+                a = make_double2(__ldcg(sa).y, 0.0);
+                b = make_double2(__ldcg(sb).y, 0.0);
             } else if (x < h) {
-                a = sa[x];
-                b = sb[x];
+                a = __ldcg(sa + x);
+                b = __ldcg(sb + x);
             } else {
-                a = cconj(sa[n - x]);
-                b = cconj(sb[n - x]);
+                a = cconj(__ldcg(sa + n - x));
+                b = cconj(__ldcg(sb + n - x));
             }
             d[e] = on ? make_double2(a.x - b.y, -(a.y + b.x)) : make_double2(0.0, 0.0);   // conj(a + i b)
         }

@@ -40,3 +40,23 @@ def test_solve_scales_by_powers_of_two(n0, J):
     for k in (400, -400, -880):
         assert np.array_equal(psi_of(n0, J, f * 2.0 ** k), psi * 2.0 ** k), k
     assert not psi_of(n0, J, np.zeros((n, n))).any()
+
+
+@pytest.mark.parametrize("case,tile", [(dict(n0=8, J=4, eps=1e-3, p=4), "0"), (dict(n0=16, J=5, eps=1e-4, p=2), "0"),
+                                       (dict(n0=16, J=7, eps=1e-4, p=2), None)])
+def test_repeated_runs_are_bit_identical(case, tile, monkeypatch):
+    """The solve right after the level-by-level reconstruction (the default
+    beyond 1024^2), on memory that earlier runs have used: the same values
+    every time."""
+    if tile is not None:
+        monkeypatch.setenv("WRC_RECON_TILE", tile)
+    v = W.fujiwhara_small().vortices
+    out = []
+    for _ in range(4):
+        with B.Run(W.RunParams(re=5000.0, **case)) as run:
+            run.init_vortices(v)
+            run.step(3)
+            run.sync()
+            out.append(run.active())
+    for idx, om in out[1:]:
+        assert np.array_equal(idx, out[0][0]) and np.array_equal(om, out[0][1])
