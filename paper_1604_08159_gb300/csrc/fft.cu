@@ -135,7 +135,9 @@ __device__ __forceinline__ void dft(C (&u)[R]) {
 }
 
 // Shared-memory index with one pad slot per 16 (spreads the strided writes
-// of the early passes over the banks).
+// of the early passes over the banks).  For a < q, q a power of two,
+// pad(a + r q) = pad(a) + pad(r q): the second term is the same for every
+// thread of a block, and not computed per access.
 __device__ __forceinline__ int pad(int x) { return x + (x >> 4); }
 
 template <int N> struct Log2;
@@ -159,6 +161,7 @@ template <int E, int R, bool INV, typename C>
 __device__ __forceinline__ void radix_pass(C (&v)[E], C* sm, int i, int nt, int p, const C* __restrict__ ptw,
                                            bool last) {
     constexpr int G = E / R;
+    const int pi = pad(i);
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         const int b = i + nt * g;
@@ -179,15 +182,15 @@ __device__ __forceinline__ void radix_pass(C (&v)[E], C* sm, int i, int nt, int 
 #pragma unroll
             for (int r = 0; r < R; ++r) v[g + r * G] = u[r];
         } else {
-            const int base = (b - k) * R + k;
+            const int wb = pad((b - k) * R + k);
 #pragma unroll
-            for (int r = 0; r < R; ++r) sm[pad(base + r * p)] = u[r];
+            for (int r = 0; r < R; ++r) sm[wb + pad(r * p)] = u[r];
         }
     }
     if (!last) {
         __syncthreads();
 #pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = sm[pad(i + e * nt)];
+        for (int e = 0; e < E; ++e) v[e] = sm[pi + pad(e * nt)];
         __syncthreads();
     }
 }
@@ -209,6 +212,7 @@ __device__ __forceinline__ void fft_reg(C (&v)[E], C* sm, int i, int n, int logn
         logp += Log2<R0>::v;
     }
     const int npass = (logn - logp) / Log2<E>::v;
+#pragma unroll 1
     for (int q = 0; q < npass; ++q) {
         radix_pass<E, E, INV>(v, sm, i, nt, p, ptw, q == npass - 1);
         if (p > 1) ptw += E * p;
@@ -313,8 +317,13 @@ __global__ void __launch_bounds__(256) k_px_fwd(const T* __restrict__ Rf, cx_t<T
 // (-d(kx) d(ky) + i (sigma(kx) - sigma(ky))/2) X1 and
 // (d(kx) d(ky) + i (sigma(c2) - sigma(ky))/2) X2.  Each is inverse-transformed
 // along y into row c of QT / WT (n x n).
-template <typename T, int E, int R0, bool QW>
-__global__ void __launch_bounds__(256) k_py_solve(cx_t<T>* __restrict__ ST, cx_t<T>* __restrict__ QT,
+// LOOP: one copy of the passes' code serves the transforms in turn; else each
+// output has its own.  Measured, mixed runs: 48 members of 256^2 .. 2048^2
+// take 8.55 ms a step with own copies and 7.84 with one (the instruction
+// caches hold it; the kernel at 256^2 first-run 41 us and 22); at 4096^2,
+// where a launch amortises its fetches, own copies take 216 us and one 250.
+template <typename T, int E, int R0, bool QW, bool LOOP>
+__global__ void __launch_bounds__(256, 2) k_py_solve(cx_t<T>* __restrict__ ST, cx_t<T>* __restrict__ QT,
                                                   cx_t<T>* __restrict__ WT, int n, int logn,
                                                   const cx_t<T>* __restrict__ tw, const T* __restrict__ sigma,
                                                   const T* __restrict__ dsym, T scale, int want_psi) {
@@ -328,99 +337,102 @@ __global__ void __launch_bounds__(256) k_py_solve(cx_t<T>* __restrict__ ST, cx_t
     const bool on = kx < h;
     const int kxs = on ? kx : 0;
     // exchange buffer of the FFT passes; with QW the forward spectrum keeps a
-    // buffer of its own (F(ky) in natural order), from which every output
-    // recomputes its values instead of holding them in registers
+    // buffer of its own (in natural order), from which every output takes its
+    // values instead of holding them in registers
     C* sm = (C*)smraw + (size_t)f * (QW ? 2 : 1) * smlen_of(n);
     C* fb = QW ? sm + smlen_of(n) : sm;
     C* row = ST + (size_t)kxs * n;
+    const int c2 = kxs == 0 ? h : n - kxs;
+    const T sx = sigma[kxs], sh = sigma[h], dx = QW ? dsym[kxs] : T(0), sc2 = sigma[c2];
+    // Transforms in turn: the forward one, psi's, and with QW those of
+    // U + i V and of S11 + i S12 for columns kx and c2.
+    enum { kForward, kPsi, kUV1, kUV2, kS1, kS2, kEnd };
     C v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = on ? row[i + e * nt] : mk<C>(T(0), T(0));
-    fft_reg<E, R0, false>(v, sm, i, n, logn, tw);
-#pragma unroll
-    for (int e = 0; e < E; ++e) fb[pad(i + e * nt)] = v[e];
-    __syncthreads();
-    const T sx = sigma[kxs], sh = sigma[h];
-    // X1, X2 at ky from the forward spectrum (see above)
-    auto x12 = [&](int ky, C& a, C& b) {
-        const C fk = fb[pad(ky)];
-        const C fm = cconj(fb[pad((n - ky) & (n - 1))]);
-        const T sy = sigma[ky];
+    // the values of output o, conjugated: an inverse transform is conj FFT
+    // conj, bit for bit
+    const auto prepare = [&](int o) {
+        const bool second = o == kUV2 || o == kS2;
         if (kxs == 0) {
-            const C s = cadd(fk, fm), d = csub(fk, fm);
-            const T f0 = ky == 0 ? T(0) : scale / (sx + sy);
-            const T fn = scale / (sh + sy);
-            a = cscale(s, T(0.5) * f0);
-            b = mk<C>(T(0.5) * fn * d.y, T(-0.5) * fn * d.x);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {   // conj of psi's X1 + i X2, else of X1 or X2
+                const int ky = i + e * nt;
+                const C fk = fb[pad(ky)], fm = cconj(fb[pad((n - ky) & (n - 1))]);
+                const C s = cadd(fk, fm), d = csub(fk, fm);
+                const T f0 = ky == 0 ? T(0) : scale / (sx + sigma[ky]);
+                const T fn = scale / (sh + sigma[ky]);
+                const C a = cscale(s, T(0.5) * f0), b = mk<C>(T(0.5) * fn * d.y, T(-0.5) * fn * d.x);
+                v[e] = cconj(o == kPsi ? mk<C>(a.x - b.y, a.y + b.x) : (second ? b : a));
+            }
         } else {
-            const T fc = scale / (sx + sy);
-            a = cscale(fk, fc);
-            b = cscale(fm, fc);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                const int ky = i + e * nt;
+                const C x = fb[second ? pad((n - ky) & (n - 1)) : pad(i) + pad(e * nt)];
+                v[e] = second ? x : cconj(x);
+            }
+        }
+        if constexpr (QW) {
+            if (o != kPsi) {
+                // the multiplier's conj: (mr + mrd d(ky), -(mid d(ky) + mi - mis sigma(ky)))
+                const bool uv = o < kS1;
+                const T sg = second ? -dx : dx;
+                const T mr = uv ? sg : T(0), mrd = uv ? T(0) : -sg, mid = uv ? T(-1) : T(0);
+                const T mi = uv ? T(0) : T(-0.5) * (second ? sc2 : sx), mis = uv ? T(0) : T(0.5);
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int ky = i + e * nt;
+                    const T dk = dsym[ky];
+                    v[e] = cmul(v[e], mk<C>(fma(mrd, dk, mr), fma(mid, dk, fma(mis, sigma[ky], mi))));
+                }
+            }
         }
     };
-    // psi: X1 (kx > 0) or X1 + i X2 (packed kx = 0, n/2); a step of the FP32
-    // form (want_psi 0, uniform over the grid) reads U and V, not psi
-    if (!QW || want_psi) {
+    const auto transform = [&](int o) {
+        fft_reg<E, R0, false>(v, sm, i, n, logn, tw);
+        if (o == kForward) {
+            // X1 for kx > 0 (the symbol is even in ky: X2 is conj X1(n - ky));
+            // the packed column as it is
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-            C a, b;
-            x12(i + e * nt, a, b);
-            v[e] = kxs == 0 ? mk<C>(a.x - b.y, a.y + b.x) : a;
+            for (int e = 0; e < E; ++e) {
+                const int ky = i + e * nt;
+                fb[pad(i) + pad(e * nt)] = kxs == 0 ? v[e] : cscale(v[e], scale / (sx + sigma[ky]));
+            }
+            __syncthreads();
+        } else if (on) {
+            C* dst = o == kPsi ? row : (o < kS1 ? QT : WT) + (size_t)(o == kUV1 || o == kS1 ? kxs : c2) * n;
+#pragma unroll
+            for (int e = 0; e < E; ++e) dst[i + e * nt] = cconj(v[e]);
         }
-        if constexpr (!QW) __syncthreads();   // fb is the exchange buffer
-        fft_reg<E, R0, true>(v, sm, i, n, logn, tw);
-        if (on)
-#pragma unroll
-            for (int e = 0; e < E; ++e) row[i + e * nt] = v[e];
-    }
-    if constexpr (QW) {
-        const int c2 = kxs == 0 ? h : n - kxs;
-        const T dx = dsym[kxs], sc2 = sigma[c2];
-        // U + i V, columns c1 = kx and c2
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            C a, b;
-            x12(i + e * nt, a, b);
-            v[e] = cmul(a, mk<C>(dx, dsym[i + e * nt]));
+    };
+    if constexpr (QW && !LOOP) {
+        transform(kForward);
+        // a step of the FP32 form (want_psi 0, uniform over the grid) reads U and V, not psi
+        if (want_psi) {
+            prepare(kPsi);
+            transform(kPsi);
         }
-        fft_reg<E, R0, true>(v, sm, i, n, logn, tw);
-        if (on)
-#pragma unroll
-            for (int e = 0; e < E; ++e) QT[(size_t)kxs * n + i + e * nt] = v[e];
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            C a, b;
-            x12(i + e * nt, a, b);
-            v[e] = cmul(b, mk<C>(-dx, dsym[i + e * nt]));
-        }
-        fft_reg<E, R0, true>(v, sm, i, n, logn, tw);
-        if (on)
-#pragma unroll
-            for (int e = 0; e < E; ++e) QT[(size_t)c2 * n + i + e * nt] = v[e];
+        prepare(kUV1);
+        transform(kUV1);
+        prepare(kUV2);
+        transform(kUV2);
         if (WT) {
-            // S11 + i S12
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int ky = i + e * nt;
-                C a, b;
-                x12(ky, a, b);
-                v[e] = cmul(a, mk<C>(-dx * dsym[ky], T(0.5) * (sx - sigma[ky])));
-            }
-            fft_reg<E, R0, true>(v, sm, i, n, logn, tw);
-            if (on)
-#pragma unroll
-                for (int e = 0; e < E; ++e) WT[(size_t)kxs * n + i + e * nt] = v[e];
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int ky = i + e * nt;
-                C a, b;
-                x12(ky, a, b);
-                v[e] = cmul(b, mk<C>(dx * dsym[ky], T(0.5) * (sc2 - sigma[ky])));
-            }
-            fft_reg<E, R0, true>(v, sm, i, n, logn, tw);
-            if (on)
-#pragma unroll
-                for (int e = 0; e < E; ++e) WT[(size_t)c2 * n + i + e * nt] = v[e];
+            prepare(kS1);
+            transform(kS1);
+            prepare(kS2);
+            transform(kS2);
+        }
+    } else {
+        const int end = !QW ? kUV1 : (WT ? kEnd : kS1);
+#pragma unroll 1
+        for (int o = kForward;;) {
+            transform(o);
+            if (QW && gridDim.y > 1) o = o == kForward ? kUV1 + (int)blockIdx.y : end;   // (want_psi 0)
+            else o = o == kForward && QW && !want_psi ? kUV1 : o + 1;
+            if (o == end) break;
+            prepare(o);
+            if constexpr (!QW) __syncthreads();   // fb is the exchange buffer
         }
     }
     pdl_trigger();
@@ -610,14 +622,19 @@ bool poison_rows() {
 
 template <typename T, int E, int R0>
 struct Shape {
+    static constexpr bool kOwn = E == 16 && R0 == 1;   // 4096^2 is of this shape (k_py_solve's LOOP)
+
     static int setup() {
         int bad = 0;
         bad |= cudaFuncSetAttribute(k_px_fwd<T, E, R0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
-        bad |= cudaFuncSetAttribute(k_py_solve<T, E, R0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        bad |= cudaFuncSetAttribute(k_py_solve<T, E, R0, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     kMaxSmem);
         bad |= cudaFuncSetAttribute(k_px_inv_real<T, E, R0>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
         if constexpr (std::is_same<T, float>::value) {
-            bad |= cudaFuncSetAttribute(k_py_solve<T, E, R0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            if constexpr (kOwn)
+                bad |= cudaFuncSetAttribute(k_py_solve<T, E, R0, true, false>,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem);
+            bad |= cudaFuncSetAttribute(k_py_solve<T, E, R0, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         kMaxSmem);
             bad |= cudaFuncSetAttribute(k_px_inv_pair<T, E, R0>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         kMaxSmem);
@@ -649,9 +666,16 @@ struct Shape {
             if (uv) {
                 C* QT = C2;                    // n x n
                 C* WT = st ? C3 : nullptr;     // n x n
-                { launch_pdl(k_py_solve<T, E, R0, true>, b_half, thr, 2 * smem, s, ST, QT, WT, n, logn, tw,
-                                                                        (const T*)p.sigma, (const T*)p.dsym,
-                                                                        scale, rows ? 0 : 1); note_launch(); }
+                // a step's outputs by blocks of their own, each with its own forward
+                // transform, while the lattice leaves SMs idle otherwise
+                const dim3 grid(b_half, rows && n <= 512 ? (st ? 4 : 2) : 1);
+                const auto solve = [&](auto kern) {
+                    launch_pdl(kern, grid, thr, 2 * smem, s, ST, QT, WT, n, logn, tw, (const T*)p.sigma,
+                               (const T*)p.dsym, scale, rows ? 0 : 1);
+                };
+                if constexpr (kOwn) solve(logn >= 12 ? k_py_solve<T, E, R0, true, false> : k_py_solve<T, E, R0, true, true>);
+                else solve(k_py_solve<T, E, R0, true, true>);
+                note_launch();
                 // psi: a step (rows given) reads U and V, not psi
                 if (!rows) {
                     { launch_pdl(k_transpose<C>, g_hn, tb, 0, s, ST, S, h, n); note_launch(); }
@@ -671,7 +695,7 @@ struct Shape {
                 return;
             }
         }
-        { launch_pdl(k_py_solve<T, E, R0, false>, b_half, thr, smem, s, ST, nullptr, nullptr, n, logn, tw,
+        { launch_pdl(k_py_solve<T, E, R0, false, true>, b_half, thr, smem, s, ST, nullptr, nullptr, n, logn, tw,
                                                                  (const T*)p.sigma, (const T*)p.dsym,
                                                                  scale, 1); note_launch(); }
         { launch_pdl(k_transpose<C>, g_hn, tb, 0, s, ST, S, h, n); note_launch(); }

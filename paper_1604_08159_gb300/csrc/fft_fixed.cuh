@@ -124,6 +124,7 @@ template <int E, int R>
 __device__ __forceinline__ void fx_pass(I2 (&v)[E], int& ex, I2* sm, int i, int nt, int p, const int4* __restrict__ ptw,
                                         bool last, FxShare& h) {
     constexpr int G = E / R;
+    const int pi = pad(i);
     unsigned big = 0;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -143,10 +144,10 @@ __device__ __forceinline__ void fx_pass(I2 (&v)[E], int& ex, I2* sm, int i, int 
 #pragma unroll
             for (int r = 0; r < R; ++r) v[g + r * G] = u[r];
         } else {
-            const int base = (b - k) * R + k;
+            const int wb = pad((b - k) * R + k);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                sm[pad(base + r * p)] = u[r];
+                sm[wb + pad(r * p)] = u[r];
                 big |= fx_mag(u[r]);
             }
         }
@@ -159,7 +160,7 @@ __device__ __forceinline__ void fx_pass(I2 (&v)[E], int& ex, I2* sm, int i, int 
         ex -= s;
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-            const I2 a = sm[pad(i + e * nt)];
+            const I2 a = sm[pi + pad(e * nt)];
             v[e].x = fx_shift(a.x, s);
             v[e].y = fx_shift(a.y, s);
         }
