@@ -888,6 +888,7 @@ wrc_status krylov_rosenbrock(wrc_run* R) {
     a.part = R->rbpart.as<double>();
     a.coef = R->rbsmall.as<double>();
     a.sc = a.coef + 32;
+    a.count = reinterpret_cast<unsigned*>(a.coef + 40);
     a.H = R->K.H;
     a.y = R->K.y;
     a.beta = R->K.beta;
@@ -906,16 +907,16 @@ wrc_status krylov_rosenbrock(wrc_run* R) {
     double* scr = R->fp32 ? lattice_scratch(R) : nullptr;
     if (R->fp32 && !scr) return fail(R, WRC_ERR_OOM, "lattice scratch");
     CK(cudaMemsetAsync(R->K.H, 0, sizeof(double) * (m + 1) * m, s));
+    CK(cudaMemsetAsync(a.count, 0, sizeof(unsigned), s));
     CK(rb_gradient<T>(a, s));
     // b = A_n omega + g = F(omega^n), then beta and v_0
     launch_matvec<T>((const T*)R->L, meta, n, R->Ua.as<T>(), R->Va.as<T>(),
                      R->cfg.sgs == WRC_SGS_DYNAMIC ? R->ga.as<T>() : nullptr, a.nu, a.r, (T*)a.w, g, nullptr, 0, s);
     CKL("rosenbrock b");
-    CK(rb_reduce<T>(a, 0, true, 3, -1, s));
-    CK(rb_scale<T>(a, -1, s));
+    CK(rb_pass<T>(a, 3, -1, s));
+    CK(rb_scale<T>(a, -1, s));   // also scatters q_0 to the lattice
     for (int j = 0; j < m; ++j) {
         // R(q_j) on the lattice (its ghost values included), psi[q_j], U[q_j], V[q_j]
-        launch_scatter<T>(meta, R->basis.as<T>() + (size_t)j * R->cap, n, Lq, s);
         launch_reconstruct<T>(Lq, R->act, g, s);
         if (R->fp32) {
             // spectral U, V (as in the freeze): U into the second half of the
@@ -931,12 +932,7 @@ wrc_status krylov_rosenbrock(wrc_run* R) {
             launch_velocity_active<T>((const T*)R->psi, meta, n, Uq, Vq, g, s);
         }
         CKL("rosenbrock jacobian");
-        CK(rb_apply<T>(a, j, s));
-        CK(rb_reduce<T>(a, j + 1, true, 0, j, s));
-        CK(rb_axpy<T>(a, j + 1, j, s));
-        CK(rb_reduce<T>(a, j + 1, false, 1, j, s));
-        CK(rb_axpy<T>(a, j + 1, j, s));
-        CK(rb_reduce<T>(a, 0, true, 2, j, s));
+        for (int mode = 0; mode < 3; ++mode) CK(rb_pass<T>(a, mode, j, s));
         CK(rb_scale<T>(a, j, s));
     }
     CK(rb_finish<T>(a, s));

@@ -144,6 +144,7 @@ struct RbArgs {
     double* part;           // kRbPartBlocks x (kNV + 1) partial sums
     double* coef;           // Gram-Schmidt coefficients of a pass
     double* sc;             // [0] normalisation, [1] |A q_j|^2
+    unsigned* count;        // blocks of a reduction that have finished (0 between launches)
     double* H;              // (m + 1) x m row-major
     double* y;
     double* beta;
@@ -155,12 +156,11 @@ struct RbArgs {
 constexpr int kRbPartBlocks = 1024;   // blocks of a reduction (partial-sum rows)
 constexpr int kRbPartWidth = 33;      // partial sums per block
 template <typename T> cudaError_t rb_gradient(const RbArgs& a, cudaStream_t s);
-template <typename T> cudaError_t rb_apply(const RbArgs& a, int j, cudaStream_t s);
-// Dot products of w with basis vectors 0..nv-1 (and |w|^2 with self), reduced,
-// then the bookkeeping of `mode` (0: first Gram-Schmidt pass of step j, 1:
-// second pass, 2: norm and breakdown test of step j, 3: beta).
-template <typename T> cudaError_t rb_reduce(const RbArgs& a, int nv, bool self, int mode, int j, cudaStream_t s);
-template <typename T> cudaError_t rb_axpy(const RbArgs& a, int nv, int j, cudaStream_t s);
+// One launch: w from the operator (mode 0: the first Gram-Schmidt pass of
+// step j) or w -= Q coef (1: the second pass; 2: the norm and breakdown test),
+// or w as it is (3: beta); then its dot products with basis vectors 0..j
+// (modes 0 and 1) and |w|^2, and their bookkeeping.
+template <typename T> cudaError_t rb_pass(const RbArgs& a, int mode, int j, cudaStream_t s);
 template <typename T> cudaError_t rb_scale(const RbArgs& a, int j, cudaStream_t s);
 // phi_1 of the projected matrix and the update of omega (and L).
 template <typename T> cudaError_t rb_finish(const RbArgs& a, cudaStream_t s);

@@ -6,10 +6,14 @@
 // Poisson solve per Krylov vector, so the Arnoldi process runs as a sequence
 // of launches driven by the host (api.cu) rather than inside the persistent
 // kernel.  Gram-Schmidt is applied twice (classical), with FP64 inner
-// products accumulated per block and added in a fixed order; the Krylov
+// products accumulated per block and added in a fixed order, each pass one
+// launch with the operator or the update before it and the bookkeeping after
+// it (k_rb_pass); the Krylov
 // dimension used (a happy breakdown stops it) lives on the device, and every
 // kernel of a later Arnoldi step returns at once.  phi_1 and the update as in
 // the persistent kernel.
+#include <algorithm>
+
 #include "krylov_impl.cuh"
 
 namespace wrc {
@@ -17,6 +21,7 @@ namespace wrc {
 namespace {
 
 constexpr int kRbThreads = 256;
+constexpr int kRbPts = 128;            // threads, and points of a turn, of a k_rb_pass block
 constexpr int kRbMaxVec = kNV + 1;   // basis vectors of a pass, and w itself
 static_assert(kRbMaxVec == kRbPartWidth, "partial-sum rows");
 
@@ -32,132 +37,206 @@ __global__ void k_rb_grad(const T* __restrict__ F, const uint32_t* __restrict__ 
     }
 }
 
-// w = A_n q - U[q] D_x omega - V[q] D_y omega (F holds R(q) with its ghosts).
-template <typename T, int P>
-__global__ void k_rb_apply(const T* __restrict__ F, const uint32_t* __restrict__ meta, int n,
-                           const T* __restrict__ Ua, const T* __restrict__ Va, T nu, T r,
-                           const T* __restrict__ Uq, const T* __restrict__ Vq, const T* __restrict__ dwx,
-                           const T* __restrict__ dwy, T* __restrict__ w, Geom g, T c1J, T c2J,
-                           const int* __restrict__ kstop, int j) {
-    if (j >= *kstop) return;
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x)
-        w[a] = apply_point<T, false, P>(F, meta[a], Ua[a], Va[a], nu, r, g, c1J, c2J) - Uq[a] * dwx[a] -
-               Vq[a] * dwy[a];
-}
-
-// Per-block FP64 partial sums: part[b * kRbMaxVec + v] = sum over the block's
-// points of basis_v . w for v < nv, and (self) |w|^2 at v = nv.
-template <typename T>
-__global__ void __launch_bounds__(kRbThreads) k_rb_dots(const T* __restrict__ basis, long long ld, int nv,
-                                                        const T* __restrict__ w, int n, bool self,
-                                                        double* __restrict__ part, const int* __restrict__ kstop,
-                                                        int j) {
-    if (j >= *kstop) return;
-    __shared__ double s_red[kRbThreads / 32][kRbMaxVec];
-    double acc[kRbMaxVec];
-#pragma unroll
-    for (int v = 0; v < kRbMaxVec; ++v) acc[v] = 0.0;
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x) {
-        const double x = (double)w[a];
-#pragma unroll
-        for (int v = 0; v < kRbMaxVec - 1; ++v)
-            if (v < nv) acc[v] += (double)basis[(size_t)v * ld + a] * x;
-        if (self) acc[kRbMaxVec - 1] += x * x;
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int v = 0; v < kRbMaxVec; ++v) {
-        double s = acc[v];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) s_red[wid][v] = s;
-    }
-    __syncthreads();
-    for (int v = threadIdx.x; v < kRbMaxVec; v += blockDim.x) {
-        double s = 0.0;
-        for (int q = 0; q < kRbThreads / 32; ++q) s += s_red[q][v];
-        part[(size_t)blockIdx.x * kRbMaxVec + v] = s;
-    }
-}
-
-// Coefficient bookkeeping of one reduction (one block of 64 threads; the
-// partial sums of nblk blocks added in block order):
-//   mode 0 (first pass of step j): c = Q^T w -> H[:, j] = c, coef = c, and
-//          |A q_j|^2 = |w|^2 kept for the breakdown test;
-//   mode 1 (second pass): c = Q^T w -> H[:, j] += c, coef = c;
-//   mode 2 (norm after step j): h = |w|, H[j + 1][j] = h; a happy breakdown
+// What precedes a reduction of step j, the reduction, and its bookkeeping:
+//   mode 0 (first pass): w = A_n q_j - U[q_j] D_x omega - V[q_j] D_y omega
+//          (Lq holds R(q_j) with its ghosts); c = Q^T w -> H[:, j] = c,
+//          coef = c, and |A q_j|^2 = |w|^2 kept for the breakdown test;
+//   mode 1 (second pass): w -= Q coef; c = Q^T w -> H[:, j] += c, coef = c;
+//   mode 2 (norm): w -= Q coef; h = |w|, H[j + 1][j] = h; a happy breakdown
 //          (h <= tol |A q_j|) or a non-finite h stops the process at
 //          k = j + 1 (non-finite also raises flags bit 0), else scale = 1/h;
-//   mode 3 (beta): beta = |w| (b); beta = 0 stops it at k = 0, else scale = 1/beta.
+//   mode 3 (beta): beta = |w| (w = b); beta = 0 stops it at k = 0, else
+//          scale = 1/beta.
 // sc: [0] scale, [1] |A q_j|^2.
-__global__ void k_rb_sum(const double* __restrict__ part, int nblk, int nv, int mode, int j, int m, double tol,
-                         double* __restrict__ H, double* __restrict__ coef, double* __restrict__ sc,
-                         double* __restrict__ beta, int* __restrict__ kstop, int* __restrict__ flags) {
-    if (mode != 3 && j >= *kstop) return;
-    __shared__ double s_out[kRbMaxVec];
-    const int nout = (mode == 2 || mode == 3) ? 1 : nv + (mode == 0 ? 1 : 0);
-    for (int t = threadIdx.x; t < nout; t += blockDim.x) {
-        const int v = (mode == 2 || mode == 3 || t == nv) ? kRbMaxVec - 1 : t;
-        double s = 0.0;
-        for (int b = 0; b < nblk; ++b) s += part[(size_t)b * kRbMaxVec + v];
-        s_out[t] = s;
-    }
-    __syncthreads();
-    if (mode == 0 || mode == 1) {
-        for (int t = threadIdx.x; t < nv; t += blockDim.x) {
-            const double c = s_out[t];
-            coef[t] = c;
-            H[(size_t)t * m + j] = mode == 0 ? c : H[(size_t)t * m + j] + c;
-        }
-        if (mode == 0 && threadIdx.x == 0) sc[1] = s_out[nv];
-        return;
-    }
-    if (threadIdx.x != 0) return;
-    const double q = s_out[0];
-    const double h = sqrt(q);
-    if (mode == 3) {
-        *beta = h;
-        if (!(h > 0.0) || !isfinite(h)) {
-            if (!isfinite(h)) atomicOr(flags, 1);
-            *kstop = 0;
-            sc[0] = 0.0;
-        } else {
-            *kstop = m;
-            sc[0] = 1.0 / h;
-        }
-        return;
-    }
-    H[(size_t)(j + 1) * m + j] = h;
-    const bool bad = !isfinite(h) || !isfinite(sc[1]);
-    if (bad) atomicOr(flags, 1);
-    if (bad || h <= tol * sqrt(sc[1])) *kstop = j + 1;
-    else sc[0] = 1.0 / h;
-}
-
-// w -= sum_{v < nv} coef_v basis_v (in the bulk type).
-template <typename T>
-__global__ void k_rb_axpy(const T* __restrict__ basis, long long ld, int nv, const double* __restrict__ coef,
-                          T* __restrict__ w, int n, const int* __restrict__ kstop, int j) {
-    if (j >= *kstop) return;
+//
+// Bound by FP64 issue (one warp instruction per ~65 cycles and SM
+// sub-partition): a block takes 128 points, its points' products with vector
+// v go to warp v mod 4, four to a lane, and the lanes' sums of eight vectors
+// are joined in nine exchanges instead of 8 x 5.  The block that finishes
+// last adds the blocks' sums in block order.  One launch for what took three
+// (the operator or update, the dots with every vector's 32-lane sums, one
+// block's serial sums): 16.9K points of 512^2, m = 31, a vector's launches
+// beside its reconstruction and solve 100 -> 20 us, the 31 vectors 4.97 ->
+// 2.50 ms.
+template <typename T, int P>
+__global__ void __launch_bounds__(kRbPts) k_rb_pass(RbArgs A, int mode, int j) {
+    pdl_wait();
+    if (mode != 3 && j >= *(const volatile int*)A.kstop) return;
+    __shared__ double s_w[kRbPts];
+    __shared__ double s_red[kRbPts / 32][32];
     __shared__ T s_c[kNV];
-    for (int t = threadIdx.x; t < nv; t += blockDim.x) s_c[t] = (T)coef[t];
+    __shared__ int s_last;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, n = A.n;
+    const int nv = mode == 3 ? 0 : j + 1, ndot = mode <= 1 ? nv : 0;
+    const T* basis = (const T*)A.basis;
+    T* w = (T*)A.w;
+    if (mode == 1 || mode == 2)
+        for (int t = tid; t < nv; t += kRbPts) s_c[t] = (T)A.coef[t];
     __syncthreads();
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x) {
-        T p[4] = {T(0), T(0), T(0), T(0)};
-        for (int v = 0; v < nv; ++v) p[v & 3] += basis[(size_t)v * ld + a] * s_c[v];
-        w[a] -= (p[0] + p[1]) + (p[2] + p[3]);
+    double acc[8], nrm = 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+    for (int base = blockIdx.x * kRbPts; base < n; base += gridDim.x * kRbPts) {
+        const int i = base + tid;
+        T x = T(0);
+        if (i < n) {
+            if (mode == 0) {
+                x = apply_point<T, false, P>((const T*)A.Lq, A.meta[i], ((const T*)A.Ua)[i], ((const T*)A.Va)[i],
+                                             (T)A.nu, (T)A.r, A.g, (T)A.c1J, (T)A.c2J) -
+                    ((const T*)A.Uq)[i] * ((const T*)A.dwx)[i] - ((const T*)A.Vq)[i] * ((const T*)A.dwy)[i];
+                w[i] = x;
+            } else {
+                x = w[i];
+                if (mode != 3) {
+                    T p[4] = {T(0), T(0), T(0), T(0)};
+                    for (int v = 0; v < nv; v += 8) {
+                        T b[8];
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) b[u] = v + u < nv ? basis[(size_t)(v + u) * A.ld + i] : T(0);
+#pragma unroll
+                        for (int u = 0; u < 8; ++u)
+                            if (v + u < nv) p[u & 3] += b[u] * s_c[v + u];
+                    }
+                    x -= (p[0] + p[1]) + (p[2] + p[3]);
+                    w[i] = x;
+                }
+            }
+        }
+        const double xd = (double)x;
+        if (mode != 1) nrm += xd * xd;
+        if (mode <= 1) {
+            s_w[tid] = xd;
+            T b[8][4];
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int v = wid + 4 * q, c = base + 32 * u + lane;
+                    b[q][u] = v < ndot && c < n ? basis[(size_t)v * A.ld + c] : T(0);
+                }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+                if (wid + 4 * q < ndot)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc[q] += (double)b[q][u] * s_w[32 * u + lane];
+            __syncthreads();
+        }
     }
+    double* part = A.part + (size_t)blockIdx.x * kRbMaxVec;
+    if (mode <= 1) {
+        // lane bits 4, 3, 2 choose the vector, the other lanes are added
+        double r4[4], r2[2], r1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const bool h = lane & 16;
+            const double send = h ? acc[q] : acc[q + 4];
+            r4[q] = (h ? acc[q + 4] : acc[q]) + __shfl_xor_sync(0xffffffffu, send, 16);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const bool h = lane & 8;
+            const double send = h ? r4[q] : r4[q + 2];
+            r2[q] = (h ? r4[q + 2] : r4[q]) + __shfl_xor_sync(0xffffffffu, send, 8);
+        }
+        {
+            const bool h = lane & 4;
+            const double send = h ? r2[0] : r2[1];
+            r1 = (h ? r2[1] : r2[0]) + __shfl_xor_sync(0xffffffffu, send, 4);
+        }
+        r1 += __shfl_xor_sync(0xffffffffu, r1, 2);
+        r1 += __shfl_xor_sync(0xffffffffu, r1, 1);
+        const int v = wid + 4 * ((lane >> 2) & 4 | (lane >> 2) & 2 | (lane >> 2) & 1);
+        if ((lane & 3) == 0 && v < ndot) part[v] = r1;
+    }
+    if (mode != 1) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+        if (lane == 0) s_red[0][wid] = nrm;
+        __syncthreads();
+        if (tid == 0) part[kRbMaxVec - 1] = (s_red[0][0] + s_red[0][1]) + (s_red[0][2] + s_red[0][3]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        s_last = atomicAdd(A.count, 1u) == gridDim.x - 1 ? 1 : 0;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) {
+        pdl_trigger();
+        return;
+    }
+    // the last block: sums over the blocks (warp q takes blocks q, q + 4, ..), then the bookkeeping
+    const int nb = gridDim.x;
+    double sum = 0.0;
+    if (mode >= 2) {
+        for (int b = tid; b < nb; b += kRbPts) sum += __ldcg(A.part + (size_t)b * kRbMaxVec + kRbMaxVec - 1);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    } else if (lane < ndot || (mode == 0 && lane == ndot)) {
+        const double* p = A.part + (lane < ndot ? lane : kRbMaxVec - 1);
+        for (int b = wid; b < nb; b += 4 * 8) {
+            double x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = b + 4 * u < nb ? __ldcg(p + (size_t)(b + 4 * u) * kRbMaxVec) : 0.0;
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (b + 4 * u < nb) sum += x[u];
+        }
+    }
+    s_red[wid][lane] = sum;
+    __syncthreads();
+    if (wid == 0) {
+        const double c = (s_red[0][lane] + s_red[1][lane]) + (s_red[2][lane] + s_red[3][lane]);
+        if (lane < ndot) {
+            A.coef[lane] = c;
+            double* h = A.H + (size_t)lane * A.m + j;
+            *h = mode == 0 ? c : *h + c;
+        }
+        if (mode == 0 && lane == ndot) A.sc[1] = c;
+        if (mode >= 2 && lane == 0) {
+            const double h = sqrt(c);
+            if (mode == 3) {
+                *A.beta = h;
+                if (!(h > 0.0) || !isfinite(h)) {
+                    if (!isfinite(h)) atomicOr(A.flags, 1);
+                    *A.kstop = 0;
+                    A.sc[0] = 0.0;
+                } else {
+                    *A.kstop = A.m;
+                    A.sc[0] = 1.0 / h;
+                }
+            } else {
+                A.H[(size_t)(j + 1) * A.m + j] = h;
+                const double q = A.sc[1];
+                const bool bad = !isfinite(h) || !isfinite(q);
+                if (bad) atomicOr(A.flags, 1);
+                if (bad || h <= A.tol * sqrt(q)) *A.kstop = j + 1;
+                else A.sc[0] = 1.0 / h;
+            }
+        }
+        if (lane == 0) *A.count = 0u;   // for the next launch
+    }
+    pdl_trigger();
 }
 
-// basis_{j + 1} = w * scale, unless the process stopped at step j.
+// basis_{j + 1} = w * scale, also into the lattice Lq, unless the process
+// stopped at step j.
 template <typename T>
-__global__ void k_rb_scale(T* __restrict__ basis, long long ld, const T* __restrict__ w, int n,
-                           const double* __restrict__ sc, const int* __restrict__ kstop, int j) {
-    if (j >= 0 && *kstop <= j + 1) return;   // stopped at or before step j
-    const double s = sc[0];
-    T* dst = basis + (size_t)(j + 1) * ld;
-    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < n; a += gridDim.x * blockDim.x)
-        dst[a] = (T)((double)w[a] * s);
+__global__ void k_rb_scale(RbArgs A, int j) {
+    pdl_wait();
+    if (j >= 0 && *(const volatile int*)A.kstop <= j + 1) return;   // stopped at or before step j
+    const double s = A.sc[0];
+    const T* w = (const T*)A.w;
+    T* dst = (T*)A.basis + (size_t)(j + 1) * A.ld;
+    T* Lq = (T*)A.Lq;
+    for (int a = blockIdx.x * blockDim.x + threadIdx.x; a < A.n; a += gridDim.x * blockDim.x) {
+        const T x = (T)((double)w[a] * s);
+        dst[a] = x;
+        Lq[meta_pos(A.meta[a])] = x;
+    }
+    pdl_trigger();
 }
 
 // y = phi_1(dt H_k) e_1 (k = *kstop; zero for k = 0), by one block.
@@ -221,39 +300,20 @@ cudaError_t rb_gradient(const RbArgs& a, cudaStream_t s) {
 }
 
 template <typename T>
-cudaError_t rb_apply(const RbArgs& a, int j, cudaStream_t s) {
+cudaError_t rb_pass(const RbArgs& a, int mode, int j, cudaStream_t s) {
+    // the last block adds this many sums, one at a time: two blocks a SM beyond 39K points
+    const int nb = std::max(1, std::min((a.n + kRbPts - 1) / kRbPts, 304));
     rb_by_order(a.g.P, [&](auto PC) {
         constexpr int P = decltype(PC)::value;
-        k_rb_apply<T, P><<<rb_blocks(a.n), kRbThreads, 0, s>>>(
-            (const T*)a.Lq, a.meta, a.n, (const T*)a.Ua, (const T*)a.Va, (T)a.nu, (T)a.r, (const T*)a.Uq,
-            (const T*)a.Vq, (const T*)a.dwx, (const T*)a.dwy, (T*)a.w, a.g, (T)a.c1J, (T)a.c2J, a.kstop, j);
+        launch_pdl(k_rb_pass<T, P>, nb, kRbPts, 0, s, a, mode, j);
     });
     note_launch();
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t rb_reduce(const RbArgs& a, int nv, bool self, int mode, int j, cudaStream_t s) {
-    const int nb = rb_blocks(a.n);
-    k_rb_dots<T><<<nb, kRbThreads, 0, s>>>((const T*)a.basis, a.ld, nv, (const T*)a.w, a.n, self, a.part, a.kstop,
-                                           mode == 3 ? -1 : j);
-    note_launch();
-    k_rb_sum<<<1, 64, 0, s>>>(a.part, nb, nv, mode, j, a.m, a.tol, a.H, a.coef, a.sc, a.beta, a.kstop, a.flags);
-    note_launch();
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t rb_axpy(const RbArgs& a, int nv, int j, cudaStream_t s) {
-    k_rb_axpy<T><<<rb_blocks(a.n), kRbThreads, 0, s>>>((const T*)a.basis, a.ld, nv, a.coef, (T*)a.w, a.n, a.kstop,
-                                                       j);
-    note_launch();
-    return cudaGetLastError();
-}
-
-template <typename T>
 cudaError_t rb_scale(const RbArgs& a, int j, cudaStream_t s) {
-    k_rb_scale<T><<<rb_blocks(a.n), kRbThreads, 0, s>>>((T*)a.basis, a.ld, (const T*)a.w, a.n, a.sc, a.kstop, j);
+    launch_pdl(k_rb_scale<T>, rb_blocks(a.n), kRbThreads, 0, s, a, j);
     note_launch();
     return cudaGetLastError();
 }
@@ -270,9 +330,7 @@ cudaError_t rb_finish(const RbArgs& a, cudaStream_t s) {
 
 #define WRC_INST(T)                                                                   \
     template cudaError_t rb_gradient<T>(const RbArgs&, cudaStream_t);                 \
-    template cudaError_t rb_apply<T>(const RbArgs&, int, cudaStream_t);               \
-    template cudaError_t rb_reduce<T>(const RbArgs&, int, bool, int, int, cudaStream_t); \
-    template cudaError_t rb_axpy<T>(const RbArgs&, int, int, cudaStream_t);           \
+    template cudaError_t rb_pass<T>(const RbArgs&, int, int, cudaStream_t);           \
     template cudaError_t rb_scale<T>(const RbArgs&, int, cudaStream_t);               \
     template cudaError_t rb_finish<T>(const RbArgs&, cudaStream_t);
 WRC_INST(double)
