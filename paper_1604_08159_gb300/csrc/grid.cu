@@ -101,12 +101,53 @@ __global__ void k_scatter(const uint32_t* __restrict__ meta, const T* __restrict
 // Pass 1: the points odd in one direction only (one 1-D prediction each),
 // the first n^2/4 indices odd rows and even columns, the next n^2/4 even rows
 // and odd columns (n = NJ / 2^(J-j) points per row at this level).
-template <typename T>
+// Order 2P = 4: four points a thread and turn, whose flags and predictor
+// points (of level j - 1, not written here) are loaded together: bound by the
+// latency of a turn's loads, not by the ~2 words a point.  Finest level of
+// 4096^2, FP32: passes 58 and 63 us one point at a time, 43 and 28 so.
+constexpr int kReconPts = 4;
+template <typename T, int P>
 __global__ void k_recon_level_1d(T* __restrict__ L, const uint8_t* __restrict__ act, int j, Geom g) {
     pdl_wait();
     const int sh = g.J - j;
     const int lh = g.L - sh - 1;             // log2(n / 2)
     const int q = 1 << (2 * lh);             // n^2 / 4
+    if constexpr (P == 2) {
+        const int stride = gridDim.x * blockDim.x, s = 1 << sh, m = g.mask;
+        for (int t0 = blockIdx.x * blockDim.x + threadIdx.x; t0 < 2 * q; t0 += kReconPts * stride) {
+            long long p[kReconPts];
+            T v[kReconPts][4];
+            bool need[kReconPts];
+#pragma unroll
+            for (int e = 0; e < kReconPts; ++e) {
+                const int t = t0 + e * stride;
+                need[e] = t < 2 * q;
+                const int tt = need[e] ? t : 0, u = tt < q ? tt : tt - q;
+                const int r = u >> lh, c = u & ((1 << lh) - 1);
+                const int k = (tt < q ? 2 * r + 1 : 2 * r) << sh;
+                const int i = (tt < q ? 2 * c : 2 * c + 1) << sh;
+                p[e] = ((long long)k << g.L) + i;
+                if (tt < q) {
+                    v[e][0] = L[((long long)((k - s) & m) << g.L) + i];
+                    v[e][1] = L[((long long)((k + s) & m) << g.L) + i];
+                    v[e][2] = L[((long long)((k - 3 * s) & m) << g.L) + i];
+                    v[e][3] = L[((long long)((k + 3 * s) & m) << g.L) + i];
+                } else {
+                    const T* row = L + ((long long)k << g.L);
+                    v[e][0] = row[(i - s) & m];
+                    v[e][1] = row[(i + s) & m];
+                    v[e][2] = row[(i - 3 * s) & m];
+                    v[e][3] = row[(i + 3 * s) & m];
+                }
+                need[e] = need[e] && !act[p[e]];
+            }
+#pragma unroll
+            for (int e = 0; e < kReconPts; ++e)
+                if (need[e]) L[p[e]] = dd4<T>(v[e][0], v[e][1], v[e][2], v[e][3]);
+        }
+        pdl_trigger();
+        return;
+    }
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < 2 * q; t += gridDim.x * blockDim.x) {
         const int u = t < q ? t : t - q;
         const int r = u >> lh, c = u & ((1 << lh) - 1);
@@ -132,26 +173,49 @@ __global__ void k_recon_level_2d(T* __restrict__ L, const uint8_t* __restrict__ 
     const int s = 1 << sh, m = g.mask;
     const int lh = g.L - sh - 1;
     const int q = 1 << (2 * lh);
+    if constexpr (P == 2) {   // as in pass 1
+        const int stride = gridDim.x * blockDim.x;
+        for (int t0 = blockIdx.x * blockDim.x + threadIdx.x; t0 < q; t0 += kReconPts * stride) {
+            T v[kReconPts][4];
+            uint8_t a[kReconPts][4];
+            bool need[kReconPts];
+#pragma unroll
+            for (int x = 0; x < kReconPts; ++x) {
+                const int t = t0 + x * stride, tt = t < q ? t : 0;
+                const int k = (2 * (tt >> lh) + 1) << sh, i = (2 * (tt & ((1 << lh) - 1)) + 1) << sh;
+                const int ks[4] = {(k - s) & m, (k + s) & m, (k - 3 * s) & m, (k + 3 * s) & m};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const long long pe = ((long long)ks[e] << g.L) + i;
+                    a[x][e] = act[pe];
+                    v[x][e] = L[pe];
+                }
+                need[x] = t < q && !act[((long long)k << g.L) + i];
+            }
+#pragma unroll
+            for (int x = 0; x < kReconPts; ++x) {
+                if (!need[x]) continue;
+                const int t = t0 + x * stride;
+                const int k = (2 * (t >> lh) + 1) << sh, i = (2 * (t & ((1 << lh) - 1)) + 1) << sh;
+                const int ks[4] = {(k - s) & m, (k + s) & m, (k - 3 * s) & m, (k + 3 * s) & m};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (a[x][e]) {
+                        const T* row = L + ((size_t)ks[e] << g.L);
+                        v[x][e] = dd4<T>(row[(i - s) & m], row[(i + s) & m], row[(i - 3 * s) & m], row[(i + 3 * s) & m]);
+                    }
+                L[((long long)k << g.L) + i] = dd4<T>(v[x][0], v[x][1], v[x][2], v[x][3]);
+            }
+        }
+        pdl_trigger();
+        return;
+    }
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < q; t += gridDim.x * blockDim.x) {
         const int r = t >> lh, c = t & ((1 << lh) - 1);
         const int k = (2 * r + 1) << sh, i = (2 * c + 1) << sh;
         const long long p = ((long long)k << g.L) + i;
         if (act[p]) continue;
-        if constexpr (P == 2) {
-            const int ks[4] = {(k - s) & m, (k + s) & m, (k - 3 * s) & m, (k + 3 * s) & m};
-            T rv[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const long long pe = ((long long)ks[e] << g.L) + i;
-                if (!act[pe]) {
-                    rv[e] = L[pe];
-                } else {
-                    const T* row = L + ((size_t)ks[e] << g.L);
-                    rv[e] = dd4<T>(row[(i - s) & m], row[(i + s) & m], row[(i - 3 * s) & m], row[(i + 3 * s) & m]);
-                }
-            }
-            L[p] = dd4<T>(rv[0], rv[1], rv[2], rv[3]);
-        } else {
+        {
             // rows k -+ (2e + 1) s: the x prediction stored there by pass 1, or
             // computed again where that point is active
             T lo[P], hi[P];
@@ -1406,10 +1470,12 @@ void launch_scatter(const uint32_t* meta, const T* vals, long long n, T* L, cuda
 template <typename T>
 void launch_recon_level(T* L, const uint8_t* act, int j, const Geom& g, cudaStream_t s) {
     const long long q = level_count(j, g) / 3;   // n^2 / 4
-    { launch_pdl(k_recon_level_1d<T>, blocks_for(2 * q), kThreads, 0, s, L, act, j, g); note_launch(); }
-    if (g.P == 3) launch_pdl(k_recon_level_2d<T, 3>, blocks_for(q), kThreads, 0, s, L, act, j, g);
-    else if (g.P == 4) launch_pdl(k_recon_level_2d<T, 4>, blocks_for(q), kThreads, 0, s, L, act, j, g);
-    else launch_pdl(k_recon_level_2d<T, 2>, blocks_for(q), kThreads, 0, s, L, act, j, g);
+    by_order(g, [&](auto p) {
+        constexpr int P = decltype(p)::value;
+        launch_pdl(k_recon_level_1d<T, P>, blocks_for(2 * q), kThreads, 0, s, L, act, j, g);
+        launch_pdl(k_recon_level_2d<T, P>, blocks_for(q), kThreads, 0, s, L, act, j, g);
+    });
+    note_launch();
     note_launch();
 }
 template <typename T>

@@ -26,8 +26,8 @@ def _lib():
     B.load()
 
 
-@pytest.mark.parametrize("n0,J", [(4, 1), (16, 4), (4, 7), (16, 6)])
-@pytest.mark.parametrize("p", [2, 3, 4])
+@pytest.mark.parametrize("n0,J,p", [(n0, J, p) for n0, J in [(4, 1), (16, 4), (4, 7), (16, 6)] for p in (2, 3, 4)] +
+                         [(32, 6, 2)])   # several turns of every thread, and the reconstruction level by level
 def test_grid_bit_exact(n0, J, p):
     prm = small_params(n0=n0, J=J, eps=1e-3, p=p)
     cfg = oracle_config(prm)
