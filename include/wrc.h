@@ -165,10 +165,10 @@ wrc_status wrc_sync(wrc_run* run, int32_t timeout_ms);
  * WRC_ERR_ARG outside the range. */
 wrc_status wrc_set_wait_limit(wrc_run* run, double seconds);
 
-/* Thread-block cluster size (1, 2 or 4) of the run's next Krylov launch on
- * its current grid.  Clusters of 2 or 4 blocks pre-add their dot sums in
- * distributed shared memory; they are used when the device can hold the
- * launch with them, the environment variable WRC_KRYLOV_CLUSTER (1 or 2,
+/* Thread-block cluster size (1 or 4) of the run's next Krylov launch on
+ * its current grid.  Clusters of four blocks pre-add their dot sums in
+ * distributed shared memory; launches of at most 96 blocks use them when the
+ * device can hold the launch with them, the environment variable WRC_KRYLOV_CLUSTER (1 or 2,
  * read at wrc_create) does not cap them, and the launch path forms them: a
  * probe launch at the device's first wrc_create and the check of the
  * device's first clustered launch switch them off for the device otherwise,
@@ -438,13 +438,13 @@ wrc_status wrc_ensemble_member(wrc_ensemble* e, int32_t member, wrc_run** run);
 /* Advance every member nsteps steps (all members need an initial condition). */
 wrc_status wrc_ensemble_step(wrc_ensemble* e, int32_t nsteps);
 
-/* Block shape of the batched Krylov kernel: threads per block (64, 128 or
- * 256) and target active points per thread (1..64). */
+/* Shape of the batched Krylov launch: (64, 128 or 256) and (1..64), whose
+ * product is the least number of active points per block: a member gets
+ * another block while each of its blocks keeps that many. */
 wrc_status wrc_ensemble_set_shape(wrc_ensemble* e, int32_t threads_per_block, int32_t points_per_thread);
 
 /* Autotuner: time the batched Krylov launch over steps_per_candidate real
- * steps for each of the 9 shapes {64,128,256} x {1,2,4} (those with at least
- * one co-resident block per member), keep the fastest and
+ * steps for each of the 9 shapes {64,128,256} x {1,2,4}, keep the fastest and
  * cache it for this process per (precision, member-count bucket,
  * active-count bucket); a cached choice is applied without stepping.  The
  * chosen shape is written to out_shape[0..1] (may be NULL). */
@@ -501,7 +501,7 @@ typedef enum { WRC_REQ_QUEUED = 0, WRC_REQ_RUNNING = 1, WRC_REQ_DONE = 2, WRC_RE
 typedef struct {
     int32_t policy;               /* wrc_serve_policy */
     int32_t max_slots;            /* resident runs at most, 1..1024 (FIFO: 1) */
-    int32_t threads_per_block;    /* batched kernel shape: 64/128/256, or 0 for the */
+    int32_t threads_per_block;    /* batched launch's shape: 64/128/256, or 0 for the */
     int32_t points_per_thread;    /* autotuned shape if one is cached, else 128 x 1 */
     double hbm_budget_bytes;      /* admission budget, > 0 (e.g. 150e9) */
 } wrc_server_config;
