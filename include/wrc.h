@@ -129,7 +129,8 @@ wrc_status wrc_init_vortices(wrc_run* run, int32_t n, const double* xc, const do
  * then transform, thresholding and adaptation as above. */
 wrc_status wrc_init_field(wrc_run* run, const double* omega_lattice, int32_t device_ptr);
 
-/* Set the adaptive grid directly: `active` (NJ*NJ bytes, 0/1) and the values
+/* Set the adaptive grid directly: `active` (NJ*NJ bytes; a point is active
+ * where its byte is not 0) and the values
  * omega_lattice (NJ*NJ, read at active points only).  The grid must contain
  * every level-0 point and be closed under DD prediction (every active point's
  * predictor points active); otherwise WRC_ERR_ARG.  No thresholding is done;

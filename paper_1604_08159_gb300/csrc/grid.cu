@@ -744,18 +744,22 @@ __global__ void k_stencil_ghost(const uint8_t* __restrict__ act, uint8_t* __rest
     pdl_trigger();
 }
 
-__global__ void k_validate_grid(const uint8_t* __restrict__ act, int* __restrict__ flag, Geom g) {
+// Checks a grid given as bytes, and turns every flag that is not 0 into 1:
+// the passes over the flags take them as bits (flag_bits, words of flags).
+__global__ void k_validate_grid(uint8_t* act, int* __restrict__ flag, Geom g) {
     pdl_wait();
     const long long N = (long long)g.NJ * g.NJ;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N;
          p += (long long)gridDim.x * blockDim.x) {
         const int i = (int)(p & g.mask), k = (int)(p >> g.L);
         const int lev = level_of(i, k, g.J);
+        const uint8_t a = act[p];
+        if (a > 1) act[p] = 1;   // (other threads ask only whether it is 0)
         if (lev == 0) {
-            if (!act[p]) atomicOr(flag, 1);
+            if (!a) atomicOr(flag, 1);
             continue;
         }
-        if (!act[p]) continue;
+        if (!a) continue;
         bool ok = true;
         for_predictor_points(i, k, lev, g, [&](int qi, int qk) {
             if (!act[((long long)qk << g.L) + qi]) ok = false;
@@ -1527,7 +1531,7 @@ void launch_stencil_ghost(const uint8_t* act, uint8_t* gho, uint8_t* JJ, const G
     });
     note_launch();
 }
-void launch_validate_grid(const uint8_t* act, int* flag, const Geom& g, cudaStream_t s) {
+void launch_validate_grid(uint8_t* act, int* flag, const Geom& g, cudaStream_t s) {
     { launch_pdl(k_validate_grid, blocks_for((long long)g.NJ * g.NJ), kThreads, 0, s, act, flag, g); note_launch(); }
 }
 void launch_compact(const uint8_t* act, const uint8_t* gho, const Geom& g, int nkeys, int* blk_counts,

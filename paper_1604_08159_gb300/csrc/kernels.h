@@ -33,7 +33,7 @@ void launch_details_adj(const uint32_t* meta, long long n, const T* L, double ep
                         uint8_t* sig, uint8_t* nxt, const Geom& g, cudaStream_t s, const int* dn = nullptr);
 void launch_closure_level(uint8_t* mask, const uint8_t* excl, int j, const Geom& g, cudaStream_t s);
 void launch_stencil_ghost(const uint8_t* act, uint8_t* gho, uint8_t* JJ, const Geom& g, cudaStream_t s);
-void launch_validate_grid(const uint8_t* act, int* flag, const Geom& g, cudaStream_t s);
+void launch_validate_grid(uint8_t* act, int* flag, const Geom& g, cudaStream_t s);
 void launch_compact(const uint8_t* act, const uint8_t* gho, const Geom& g, int nkeys, int* blk_counts,
                     int* blk_off, int* counts, int* list, cudaStream_t s);
 template <typename T>
