@@ -49,7 +49,8 @@ typedef struct wrc_run wrc_run;
 typedef enum {
     WRC_OK = 0,
     WRC_ERR_ARG = -1,            /* invalid argument or configuration */
-    WRC_ERR_OOM = -2,            /* a device allocation failed */
+    WRC_ERR_OOM = -2,            /* a device allocation failed; where a grid's arrays could not grow, the
+                                  * run has no state until a new initial condition */
     WRC_ERR_CUDA = -3,           /* a CUDA call or kernel launch failed */
     WRC_ERR_BREAKDOWN_NAN = -4,  /* a non-finite value appeared in the Arnoldi process */
     WRC_ERR_TIMEOUT = -5,        /* a bounded wait ran out */

@@ -53,8 +53,13 @@ struct DevBuf {
     cudaError_t grow(size_t need, size_t keep, cudaStream_t s) {
         if (need <= bytes) return cudaSuccess;
         void* q = nullptr;
-        cudaError_t e = cudaMalloc(&q, need);
-        if (e != cudaSuccess) return e;
+        // test switch: a growth beyond so many bytes fails as if the device were full
+        const char* lim = std::getenv("WRC_ALLOC_TEST_LIMIT");
+        cudaError_t e = lim && need > std::strtoull(lim, nullptr, 10) ? cudaErrorMemoryAllocation : cudaMalloc(&q, need);
+        if (e != cudaSuccess) {
+            cudaGetLastError();   // reported by the caller, not by the next launch's check
+            return e;
+        }
         if (p && keep) {
             e = cudaMemcpyAsync(q, p, keep, cudaMemcpyDeviceToDevice, s);
             if (e != cudaSuccess) return e;
@@ -260,7 +265,8 @@ double* lattice_scratch(wrc_run* R) {
 
 // The basis and its ghost values in global memory: for the batched and the
 // streaming Krylov launches and the Rosenbrock step (a single run's launch
-// keeps them in shared memory as long as they fit).
+// keeps them in shared memory as long as they fit).  Asked for whenever a
+// grid is set, grown or not: a growth that failed before has left none.
 wrc_status ensure_basis(wrc_run* R) {
     const size_t m = R->cfg.krylov_m;
     CK(R->basis.grow(8 * (size_t)R->cap * (m + 1), 0, R->st));   // 64-bit fixed point (or the bulk type)
@@ -268,12 +274,14 @@ wrc_status ensure_basis(wrc_run* R) {
     return WRC_OK;
 }
 
+bool wants_basis(const wrc_run* R) { return R->batched || R->cfg.scheme == WRC_SCHEME_ROSENBROCK; }
+
 wrc_status ensure_capacity(wrc_run* R, long long n) {
-    if (n <= R->cap) return WRC_OK;
+    if (n <= R->cap) return wants_basis(R) ? ensure_basis(R) : WRC_OK;
     long long c = n + n / 4 + 1024;
     c = (c + 255) / 256 * 256;
-    const int m = R->cfg.krylov_m;
     const cudaStream_t s = R->st;
+    R->layout += 1;   // first: some arrays have moved even if a later one cannot be had
     const size_t be = R->es * (size_t)c;
     // meta/omega of the current grid and the details keep their contents
     CK(R->meta[R->cur].grow(sizeof(uint32_t) * c, sizeof(uint32_t) * R->n_active, s));
@@ -290,7 +298,6 @@ wrc_status ensure_capacity(wrc_run* R, long long n) {
         CK(R->xd.grow(8 * be, 0, s));
         CK(R->xw.grow(3 * be, 0, s));
         R->xbasis.release(s);
-        CK(R->xbasis.grow(3 * be * (size_t)(m + 1), 0, s));
     }
     CK(R->det.grow(be, R->es * R->det_count, s));
     CK(R->Ua.grow(be, 0, s));
@@ -302,25 +309,23 @@ wrc_status ensure_capacity(wrc_run* R, long long n) {
     // the basis is rebuilt every step; its leading dimension changes with c
     R->basis.release(s);
     R->cap = c;
-    R->layout += 1;
-    if (R->batched || R->cfg.scheme == WRC_SCHEME_ROSENBROCK) TRY(ensure_basis(R));
-    return WRC_OK;
+    return wants_basis(R) ? ensure_basis(R) : WRC_OK;
 }
 
 wrc_status ensure_ghost_capacity(wrc_run* R, long long ng) {
-    if (ng <= R->cap_g && R->row_ready.p) return WRC_OK;   // the ready flags exist even for a grid without ghosts
+    if (ng <= R->cap_g && R->row_ready.p)   // the ready flags exist even for a grid without ghosts
+        return wants_basis(R) ? ensure_basis(R) : WRC_OK;
     long long c = ng + ng / 4 + 1024;
     c = (c + 255) / 256 * 256;
     const cudaStream_t s = R->st;
+    R->layout += 1;
     CK(R->row_len.grow(sizeof(int) * c, 0, s));
     CK(R->row_ready.grow(sizeof(int) * (c + 1), 0, s));
     CK(R->row_idx.grow(sizeof(int) * c * R->rmax, 0, s));
     CK(R->row_w.grow(sizeof(double) * c * R->rmax, 0, s));
     R->Gb.release(s);
     R->cap_g = c;
-    R->layout += 1;
-    if (R->batched || R->cfg.scheme == WRC_SCHEME_ROSENBROCK) TRY(ensure_basis(R));
-    return WRC_OK;
+    return wants_basis(R) ? ensure_basis(R) : WRC_OK;
 }
 
 // A grid rebuild in three parts.  Part 1 (device, capturable): the new grid
@@ -374,8 +379,12 @@ wrc_status rebuild_host(wrc_run* R) {
         off += R->gcount[j];
         ng += R->gcount[j];
     }
-    TRY(ensure_capacity(R, na));
-    TRY(ensure_ghost_capacity(R, ng));
+    wrc_status st = ensure_capacity(R, na);
+    if (st == WRC_OK) st = ensure_ghost_capacity(R, ng);
+    if (st != WRC_OK) {
+        R->init = false;   // the list, ghosts and counts on the device are a grid's that could not be set up
+        return st;
+    }
     R->pend_na = na;
     R->pend_ng = ng;
     return WRC_OK;
@@ -990,7 +999,6 @@ wrc_status exner_krylov(wrc_run* R) {
     CK(R->rbpart.grow(sizeof(double) * (size_t)maxb * kExPartWidth, 0, s));
     const ExArgs a = exner_args(R);
     ExKrylov K{};
-    K.basis = R->xbasis.as<double>();
     K.ld3 = 3 * R->cap;
     K.w = R->xw.as<double>();
     K.part = R->rbpart.as<double>();
@@ -1039,6 +1047,8 @@ wrc_status exner_krylov(wrc_run* R) {
         CK(launch_krylov_ex(A, a, plan, s));
         return WRC_OK;
     }
+    CK(R->xbasis.grow(3 * sizeof(double) * (size_t)R->cap * (m + 1), 0, s));
+    K.basis = R->xbasis.as<double>();
     CK(ex_krylov(a, K, blocks, s));
     return WRC_OK;
 }
