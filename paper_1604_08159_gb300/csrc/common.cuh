@@ -264,6 +264,11 @@ long long launches_total();
 // completed and its writes are visible; without the launch attribute it
 // returns at once) and pdl_trigger() after its work, which lets the
 // successor's launch begin.  Measured ~1 us saved per kernel boundary.
+// A pointer to what another kernel of the stream writes is not const
+// __restrict__ in such a kernel: that makes its loads read-only ones, valid
+// at any time as far as the compiler knows, which it may move above the wait
+// (seen in the FP64 transforms, which then read what the predecessor had yet
+// to write).  The tables made when a run is created keep it.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

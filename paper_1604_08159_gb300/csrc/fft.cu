@@ -225,7 +225,7 @@ __device__ __forceinline__ void fft_reg(C (&v)[E], C* sm, int i, int n, int logn
 // pass with sub-length p > 1 and radix R, entries w_{R p}^{r k} = tw[(r k) n / (R p)]
 // at [r p + k] (copies, so the transforms are those of the single table).
 template <typename C>
-__global__ void k_fft_pass_tables(const C* __restrict__ tw, C* __restrict__ ptw, int n, int logn, int E, int R0) {
+__global__ void k_fft_pass_tables(const C* tw, C* __restrict__ ptw, int n, int logn, int E, int R0) {
     pdl_wait();
     int p = 1, logp = 0, off = 0;
     auto table = [&](int R, int logR) {
@@ -259,7 +259,7 @@ __host__ __device__ constexpr int smlen_of(int n) { return n + n / 16 + 1; }
 // X_b[k] = -i (Z[k] - conj Z[n-k]) / 2, kept for k < n/2 in S (n x n/2), with
 // S[y][0] = X_y[0] + i X_y[n/2].
 template <typename T, int E, int R0>
-__global__ void __launch_bounds__(256) k_px_fwd(const T* __restrict__ Rf, cx_t<T>* __restrict__ S, int n, int logn,
+__global__ void __launch_bounds__(256) k_px_fwd(const T* Rf, cx_t<T>* __restrict__ S, int n, int logn,
                                                 const cx_t<T>* __restrict__ tw) {
     pdl_wait();
     using C = cx_t<T>;
@@ -446,9 +446,9 @@ __global__ void __launch_bounds__(256, 2) k_py_solve(cx_t<T>* __restrict__ ST, c
 // the list return at once; a pair is transformed independently of the
 // others, so the rows computed are the same.
 template <typename T, int E, int R0>
-__global__ void __launch_bounds__(256) k_px_inv_real(const cx_t<T>* __restrict__ S, T* __restrict__ out, int n,
+__global__ void __launch_bounds__(256) k_px_inv_real(const cx_t<T>* S, T* __restrict__ out, int n,
                                                      int logn, const cx_t<T>* __restrict__ tw,
-                                                     const int* __restrict__ rows) {
+                                                     const int* rows) {
     pdl_wait();
     using C = cx_t<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -505,9 +505,9 @@ __global__ void __launch_bounds__(256) k_px_inv_real(const cx_t<T>* __restrict__
 // pairs wanted, as for k_px_inv_real), block b transforms the rows of the
 // listed pairs b F / 2 ..., and the blocks past them return at once.
 template <typename T, int E, int R0>
-__global__ void __launch_bounds__(256) k_px_inv_pair(const cx_t<T>* __restrict__ Q, T* __restrict__ A,
+__global__ void __launch_bounds__(256) k_px_inv_pair(const cx_t<T>* Q, T* __restrict__ A,
                                                      T* __restrict__ B, int n, int logn,
-                                                     const cx_t<T>* __restrict__ tw, const int* __restrict__ rows) {
+                                                     const cx_t<T>* __restrict__ tw, const int* rows) {
     pdl_wait();
     using C = cx_t<T>;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(256) k_px_inv_pair(const cx_t<T>* __restrict__
 // rows[q] clear) of up to two lattices set to NaN after the inverse passes,
 // so that a step that read one would show it.
 template <typename T>
-__global__ void k_poison_rows(T* __restrict__ a, T* __restrict__ b, const int* __restrict__ rows, int n) {
+__global__ void k_poison_rows(T* __restrict__ a, T* __restrict__ b, const int* rows, int n) {
     pdl_wait();
     const long long N = (long long)n * n;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < N;
@@ -556,7 +556,7 @@ __global__ void k_poison_rows(T* __restrict__ a, T* __restrict__ b, const int* _
 
 // out[c][r] = in[r][c] for a rows x cols complex matrix, 32 x 32 tiles.
 template <typename C>
-__global__ void k_transpose(const C* __restrict__ in, C* __restrict__ out, int rows, int cols) {
+__global__ void k_transpose(const C* in, C* __restrict__ out, int rows, int cols) {
     pdl_wait();
     __shared__ C tile[32][33];
     const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;

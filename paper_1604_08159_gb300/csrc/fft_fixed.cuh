@@ -265,7 +265,7 @@ __global__ void k_fx_pass_tables(int4* __restrict__ ptw, int n, int logn, int lo
 }
 // inv[kx][ky] = scale / (sigma(kx) + sigma(ky)), kx <= n/2, 0 at kx = ky = 0
 // (a division is nine FP64 instructions).
-__global__ void k_fx_symbol(double* __restrict__ inv, const double* __restrict__ sigma, int n) {
+__global__ void k_fx_symbol(double* __restrict__ inv, const double* sigma, int n) {
     pdl_wait();
     const long long N = (long long)(n / 2 + 1) * n;
     const double scale = 1.0 / ((double)n * (double)n);
@@ -275,11 +275,9 @@ __global__ void k_fx_symbol(double* __restrict__ inv, const double* __restrict__
 }
 
 // Step 1 (see k_px_fwd).  In these kernels the wait for the predecessor comes
-// before anything else and its data is read by coherent loads: read-only
-// loads (of const __restrict__ pointers) may be moved above a wait that
-// follows other code, where they read what the predecessor has yet to write.
+// before anything else and its data is read by coherent loads (see launch_pdl).
 template <int E, int R0>
-__global__ void __launch_bounds__(kFxThreads) k_px_fwd_fx(const double* __restrict__ Rf, double2* __restrict__ S, int n,
+__global__ void __launch_bounds__(kFxThreads) k_px_fwd_fx(const double* Rf, double2* __restrict__ S, int n,
                                                    int logn, const int4* __restrict__ tw) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -390,9 +388,9 @@ __global__ void __launch_bounds__(kFxThreads) k_py_solve_fx(double2* __restrict_
 
 // Step 5 for psi (see k_px_inv_real).
 template <int E, int R0>
-__global__ void __launch_bounds__(kFxThreads) k_px_inv_fx(const double2* __restrict__ S, double* __restrict__ out, int n,
+__global__ void __launch_bounds__(kFxThreads) k_px_inv_fx(const double2* S, double* __restrict__ out, int n,
                                                    int logn, const int4* __restrict__ tw,
-                                                   const int* __restrict__ rows) {
+                                                   const int* rows) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ unsigned s_slot[kFxEvents];

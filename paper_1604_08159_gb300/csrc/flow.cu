@@ -81,8 +81,8 @@ void by_order(const Geom& g, F&& f) {
 }
 
 template <typename T, int P>
-__global__ void k_velocity_active(const T* __restrict__ psi, const uint32_t* __restrict__ meta, long long n,
-                                  T* __restrict__ Ua, T* __restrict__ Va, Geom g, T c1, const int* __restrict__ dn) {
+__global__ void k_velocity_active(const T* psi, const uint32_t* meta, long long n,
+                                  T* __restrict__ Ua, T* __restrict__ Va, Geom g, T c1, const int* dn) {
     pdl_wait();
     n = eff_n(dn, n);
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -111,8 +111,8 @@ __device__ __forceinline__ long long listed_point(const int* rows, long long e, 
 }
 
 template <typename T>
-__global__ void k_strain_nut(const T* __restrict__ S11, const T* __restrict__ S12, T* __restrict__ nut,
-                             T* __restrict__ a, T* __restrict__ c, long long N, T csh2, const int* __restrict__ rows,
+__global__ void k_strain_nut(const T* S11, const T* S12, T* __restrict__ nut,
+                             T* __restrict__ a, T* __restrict__ c, long long N, T csh2, const int* rows,
                              int lg) {
     pdl_wait();
     const long long tot = listed_points(rows, N, lg);
@@ -129,9 +129,9 @@ __global__ void k_strain_nut(const T* __restrict__ S11, const T* __restrict__ S1
 }
 
 template <typename T>
-__global__ void k_velocity_gather(const T* __restrict__ Ulat, const T* __restrict__ Vlat,
-                                  const uint32_t* __restrict__ meta, long long n, T* __restrict__ Ua,
-                                  T* __restrict__ Va, const int* __restrict__ dn) {
+__global__ void k_velocity_gather(const T* Ulat, const T* Vlat,
+                                  const uint32_t* meta, long long n, T* __restrict__ Ua,
+                                  T* __restrict__ Va, const int* dn) {
     pdl_wait();
     n = eff_n(dn, n);
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -145,7 +145,7 @@ __global__ void k_velocity_gather(const T* __restrict__ Ulat, const T* __restric
 
 // Pass 3: t0 = d(t3)/dy.
 template <typename T, int P>
-__global__ void k_sgs3(const T* __restrict__ t3, T* __restrict__ t0, Geom g, T c1, const int* __restrict__ rows) {
+__global__ void k_sgs3(const T* t3, T* __restrict__ t0, Geom g, T c1, const int* rows) {
     pdl_wait();
     const long long tot = listed_points(rows, (long long)g.NJ * g.NJ, g.L);
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot;
@@ -159,8 +159,8 @@ __global__ void k_sgs3(const T* __restrict__ t3, T* __restrict__ t0, Geom g, T c
 
 // Pass 4 at the active points: g = Dxx(t2) - Dyy(t2) - 4 Dx(t0).
 template <typename T, int P>
-__global__ void k_sgs4(const T* __restrict__ t2, const T* __restrict__ t0, const uint32_t* __restrict__ meta,
-                       long long n, T* __restrict__ ga, Geom g, T c1, T c2, const int* __restrict__ dn) {
+__global__ void k_sgs4(const T* t2, const T* t0, const uint32_t* meta,
+                       long long n, T* __restrict__ ga, Geom g, T c1, T c2, const int* dn) {
     pdl_wait();
     n = eff_n(dn, n);
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -186,8 +186,8 @@ __global__ void k_sgs4(const T* __restrict__ t2, const T* __restrict__ t0, const
 // reserves the warp's total.  The loop runs warp-uniformly (a lane past n
 // takes part with no points), so the warp's shuffles see all 32 lanes.
 template <int P>
-__global__ void k_sgs_halo_mark(const uint32_t* __restrict__ meta, long long n, uint8_t* __restrict__ halo,
-                                int* __restrict__ hlist, Geom g, const int* __restrict__ dn) {
+__global__ void k_sgs_halo_mark(const uint32_t* meta, long long n, uint8_t* __restrict__ halo,
+                                int* __restrict__ hlist, Geom g, const int* dn) {
     pdl_wait();
     constexpr int R = dd_reach(P);
     constexpr int W = 2 * R + 1, NB = W * W, NW = (NB + 31) / 32;
@@ -239,7 +239,7 @@ __global__ void k_sgs_halo_mark(const uint32_t* __restrict__ meta, long long n, 
 // At halo points: S11 = D_x(D_y psi), S12 = (psi_yy - psi_xx)/2,
 // nu_t = (C_s h)^2 2 sqrt(S11^2 + S12^2) (Eq. 5); t2 = 2 nu_t S12, t3 = nu_t S11.
 template <typename T, int P>
-__global__ void k_sgs_halo_products(const T* __restrict__ psi, const int* __restrict__ hlist,
+__global__ void k_sgs_halo_products(const T* psi, const int* hlist,
                                     T* __restrict__ t2, T* __restrict__ t3, Geom g, T c1, T c2, T csh2) {
     pdl_wait();
     const int nh = hlist[0];
@@ -268,9 +268,9 @@ __global__ void k_sgs_halo_products(const T* __restrict__ psi, const int* __rest
 
 // At the active points: g = Dxx(t2) - Dyy(t2) - 4 D_x(D_y t3).
 template <typename T, int P>
-__global__ void k_sgs_halo_forcing(const T* __restrict__ t2, const T* __restrict__ t3,
-                                   const uint32_t* __restrict__ meta, long long n, T* __restrict__ ga, Geom g, T c1,
-                                   T c2, const int* __restrict__ dn) {
+__global__ void k_sgs_halo_forcing(const T* t2, const T* t3,
+                                   const uint32_t* meta, long long n, T* __restrict__ ga, Geom g, T c1,
+                                   T c2, const int* dn) {
     pdl_wait();
     n = eff_n(dn, n);
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -295,7 +295,7 @@ __global__ void k_sgs_halo_forcing(const T* __restrict__ t2, const T* __restrict
 }
 
 template <typename T, int P>
-__global__ void k_lattice_uv(const T* __restrict__ psi, T* __restrict__ U, T* __restrict__ V, Geom g, T c1) {
+__global__ void k_lattice_uv(const T* psi, T* __restrict__ U, T* __restrict__ V, Geom g, T c1) {
     pdl_wait();
     const long long N = (long long)g.NJ * g.NJ;
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N;
@@ -308,7 +308,7 @@ __global__ void k_lattice_uv(const T* __restrict__ psi, T* __restrict__ U, T* __
 }
 
 template <typename T, int P>
-__global__ void k_lattice_nut(const T* __restrict__ psi, const T* __restrict__ U, T* __restrict__ nut, Geom g,
+__global__ void k_lattice_nut(const T* psi, const T* U, T* __restrict__ nut, Geom g,
                               T c1, T c2, T csh2) {
     pdl_wait();
     const long long N = (long long)g.NJ * g.NJ;
@@ -326,11 +326,11 @@ __global__ void k_lattice_nut(const T* __restrict__ psi, const T* __restrict__ U
 // each derivative along its axis at the point's stencil level j*, i.e. with
 // lattice offsets +-s, +-2s, s = 2^(J-j*), and spacing h_{j*} = s h_J.
 template <typename T, int P>
-__global__ void __launch_bounds__(kThreads) k_matvec(const T* __restrict__ F, const uint32_t* __restrict__ meta,
-                                                     long long n, const T* __restrict__ Ua,
-                                                     const T* __restrict__ Va, const T* __restrict__ ga, T nu,
+__global__ void __launch_bounds__(kThreads) k_matvec(const T* F, const uint32_t* meta,
+                                                     long long n, const T* Ua,
+                                                     const T* Va, const T* ga, T nu,
                                                      T r, T* __restrict__ w, Geom g, T c1J, T c2J,
-                                                     const int* __restrict__ kstop, int jstep) {
+                                                     const int* kstop, int jstep) {
     pdl_wait();
     if (kstop && jstep >= *kstop) return;
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThreads) k_matvec(const T* __restrict__ F, co
 // Lattice sums of R, R^2, U^2 + V^2 and |grad R|^2 (deterministic two-stage
 // reduction: per-block partials, then the last block sums them in order).
 template <typename T, int P>
-__global__ void __launch_bounds__(kThreads) k_diag(const T* __restrict__ R, const T* __restrict__ psi,
+__global__ void __launch_bounds__(kThreads) k_diag(const T* R, const T* psi,
                                                    double* __restrict__ partials, unsigned* __restrict__ counter,
                                                    double* __restrict__ out, Geom g, T c1) {
     pdl_wait();
@@ -493,7 +493,7 @@ cudaError_t launch_diag(const T* R, const T* psi, double* partials, unsigned* co
 }
 
 template <typename A, typename B>
-__global__ void k_convert(const A* __restrict__ in, B* __restrict__ out, long long n) {
+__global__ void k_convert(const A* in, B* __restrict__ out, long long n) {
     pdl_wait();
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n; t += (long long)gridDim.x * blockDim.x)
         out[t] = (B)in[t];

@@ -24,7 +24,7 @@ constexpr double kPi = 3.141592653589793238462643383279502884;
 // larger where the vorticity is small: neither is nearer to the exact value.
 constexpr int kInitCols = 256, kInitGroup = 8;
 template <typename T, int ROWS>
-__global__ void __launch_bounds__(kInitCols) k_init_vortices(T* __restrict__ L, const double* __restrict__ prm, int n,
+__global__ void __launch_bounds__(kInitCols) k_init_vortices(T* __restrict__ L, const double* prm, int n,
                                                              Geom g) {
     __shared__ double s_x[kInitGroup][kInitCols];
     __shared__ double s_y[kInitGroup][ROWS];
@@ -73,8 +73,8 @@ __device__ __forceinline__ void flag_pair(int* rows, int h, int q) {
 }
 
 template <typename T>
-__global__ void k_scatter(const uint32_t* __restrict__ meta, const T* __restrict__ vals, long long n,
-                          T* __restrict__ L, const int* __restrict__ dn, int* __restrict__ rows, int margin,
+__global__ void k_scatter(const uint32_t* meta, const T* vals, long long n,
+                          T* __restrict__ L, const int* dn, int* __restrict__ rows, int margin,
                           int lg, int mask) {
     pdl_wait();
     n = eff_n(dn, n);
@@ -107,7 +107,7 @@ __global__ void k_scatter(const uint32_t* __restrict__ meta, const T* __restrict
 // 4096^2, FP32: passes 58 and 63 us one point at a time, 43 and 28 so.
 constexpr int kReconPts = 4;
 template <typename T, int P>
-__global__ void k_recon_level_1d(T* __restrict__ L, const uint8_t* __restrict__ act, int j, Geom g) {
+__global__ void k_recon_level_1d(T* __restrict__ L, const uint8_t* act, int j, Geom g) {
     pdl_wait();
     const int sh = g.J - j;
     const int lh = g.L - sh - 1;             // log2(n / 2)
@@ -167,7 +167,7 @@ __global__ void k_recon_level_1d(T* __restrict__ L, const uint8_t* __restrict__ 
 // predicted again.  Bit-identical to the tensor-product predictor, with one 1-D
 // prediction per point instead of five for most points.
 template <typename T, int P>
-__global__ void k_recon_level_2d(T* __restrict__ L, const uint8_t* __restrict__ act, int j, Geom g) {
+__global__ void k_recon_level_2d(T* __restrict__ L, const uint8_t* act, int j, Geom g) {
     pdl_wait();
     const int sh = g.J - j;
     const int s = 1 << sh, m = g.mask;
@@ -358,7 +358,7 @@ struct RowWalk {
 // into registers before its predictions (used in phase 3), the next level's
 // grid flags during this level's predictions.
 template <typename T, int P, int PMAX>
-__global__ void __launch_bounds__(kThreads) k_recon_tiles(T* __restrict__ L, const uint8_t* __restrict__ act, Geom g,
+__global__ void __launch_bounds__(kThreads) k_recon_tiles(T* __restrict__ L, const uint8_t* act, Geom g,
                                                           ReconTiles lay) {
     extern __shared__ __align__(16) unsigned char recon_smem[];
     T* sm = reinterpret_cast<T*>(recon_smem);
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(kThreads) k_recon_tiles(T* __restrict__ L, con
 // L) or a coarser new point (written by an earlier level's launch).  The
 // other non-current points are not written.
 template <typename T>
-__global__ void k_recon_new(T* __restrict__ L, const uint8_t* __restrict__ act, const uint8_t* __restrict__ nxt,
+__global__ void k_recon_new(T* __restrict__ L, const uint8_t* act, const uint8_t* nxt,
                             int j, Geom g) {
     pdl_wait();
     const long long cnt = level_count(j, g);
@@ -540,8 +540,8 @@ __global__ void k_recon_new(T* __restrict__ L, const uint8_t* __restrict__ act, 
 // thread: the new-grid and grid flags read as 16-byte vectors (neither is
 // written here), the chunks without a new point skipped.
 template <typename T>
-__global__ void k_recon_new_fine(T* __restrict__ L, const uint8_t* __restrict__ act,
-                                 const uint8_t* __restrict__ nxt, Geom g) {
+__global__ void k_recon_new_fine(T* __restrict__ L, const uint8_t* act,
+                                 const uint8_t* nxt, Geom g) {
     pdl_wait();
     const long long N16 = (long long)g.NJ * g.NJ / 16;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N16;
@@ -565,9 +565,9 @@ __global__ void k_recon_new_fine(T* __restrict__ L, const uint8_t* __restrict__ 
 // level j and j+1 within 2^(J-j) fine cells in x and y.  All writes to the
 // masks store the value 1, so concurrent writers agree.
 template <typename T>
-__global__ void k_details_adj(const uint32_t* __restrict__ meta, long long n, const T* __restrict__ L,
+__global__ void k_details_adj(const uint32_t* meta, long long n, const T* L,
                               double eps, T* __restrict__ det, uint8_t* __restrict__ sig,
-                              uint8_t* __restrict__ nxt, Geom g, const int* __restrict__ dn) {
+                              uint8_t* __restrict__ nxt, Geom g, const int* dn) {
     pdl_wait();
     n = eff_n(dn, n);
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -647,7 +647,7 @@ __device__ __forceinline__ void mark_predictors(uint8_t* __restrict__ mask, cons
 // Closure under prediction for one level (finest first): every marked level-j
 // point marks its predictor points, except where `excl` is set.
 template <int P>
-__global__ void k_closure_level(uint8_t* __restrict__ mask, const uint8_t* __restrict__ excl, int j, Geom g) {
+__global__ void k_closure_level(uint8_t* __restrict__ mask, const uint8_t* excl, int j, Geom g) {
     pdl_wait();
     const long long cnt = level_count(j, g);
     for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < cnt;
@@ -664,7 +664,7 @@ __global__ void k_closure_level(uint8_t* __restrict__ mask, const uint8_t* __res
 // bytes, all in flight, and never the coarser points' bytes, which the pass
 // writes.
 template <int P, int V>
-__global__ void k_closure_fine(uint8_t* __restrict__ mask, const uint8_t* __restrict__ excl, Geom g) {
+__global__ void k_closure_fine(uint8_t* __restrict__ mask, const uint8_t* excl, Geom g) {
     pdl_wait();
     const long long NV = (long long)g.NJ * g.NJ / V;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < NV;
@@ -702,7 +702,7 @@ __device__ __forceinline__ unsigned flag_bits(const uint8_t* __restrict__ f, lon
 // Bound by the chains of dependent loads: the flags of all levels are read
 // before any is looked at.
 template <int V>
-__global__ void k_stencil_ghost(const uint8_t* __restrict__ act, uint8_t* __restrict__ gho,
+__global__ void k_stencil_ghost(const uint8_t* act, uint8_t* __restrict__ gho,
                                 uint8_t* __restrict__ JJ, Geom g) {
     pdl_wait();
     const long long NV = (long long)g.NJ * g.NJ / V;
@@ -797,8 +797,8 @@ __device__ __forceinline__ void keys16(const uint8_t* __restrict__ act, const ui
 
 // Counts per key of one tile of kTile = 16 kThreads points (thread t: points
 // 16 t .. 16 t + 15 of the tile), key-major into blk_counts[key][block].
-__global__ void __launch_bounds__(kThreads) k_compact_count(const uint8_t* __restrict__ act,
-                                                            const uint8_t* __restrict__ gho, Geom g, int nkeys,
+__global__ void __launch_bounds__(kThreads) k_compact_count(const uint8_t* act,
+                                                            const uint8_t* gho, Geom g, int nkeys,
                                                             int* __restrict__ blk_counts) {
     pdl_wait();
     __shared__ int s_w[kThreads / 32][kMaxKeys];
@@ -860,7 +860,7 @@ __device__ int block_excl_scan_1024(int v, int& total) {
 // more in further rounds), the bucket bases are added when written.
 constexpr int kScanChunk = 4;
 
-__global__ void __launch_bounds__(1024) k_compact_scan(const int* __restrict__ blk_counts, int nblk, int nkeys,
+__global__ void __launch_bounds__(1024) k_compact_scan(const int* blk_counts, int nblk, int nkeys,
                                                        int* __restrict__ blk_off, int* __restrict__ counts) {
     pdl_wait();
     __shared__ int s_tot[kMaxKeys];
@@ -908,10 +908,10 @@ __global__ void __launch_bounds__(1024) k_compact_scan(const int* __restrict__ b
 // block's base offset, in lattice order.
 // A tile without an entry (its counts from k_compact_count all zero, as in
 // most tiles of a large lattice) returns at once.
-__global__ void __launch_bounds__(kThreads) k_compact_scatter(const uint8_t* __restrict__ act,
-                                                              const uint8_t* __restrict__ gho, Geom g, int nkeys,
-                                                              const int* __restrict__ blk_off,
-                                                              const int* __restrict__ blk_counts,
+__global__ void __launch_bounds__(kThreads) k_compact_scatter(const uint8_t* act,
+                                                              const uint8_t* gho, Geom g, int nkeys,
+                                                              const int* blk_off,
+                                                              const int* blk_counts,
                                                               int* __restrict__ list) {
     pdl_wait();
     __shared__ int s_base[kMaxKeys];
@@ -957,9 +957,9 @@ __global__ void __launch_bounds__(kThreads) k_compact_scatter(const uint8_t* __r
 }
 
 template <typename T>
-__global__ void k_finalize(const int* __restrict__ list, long long n, const uint8_t* __restrict__ JJ,
-                           const T* __restrict__ L, uint32_t* __restrict__ meta, T* __restrict__ omega,
-                           const int* __restrict__ dn) {
+__global__ void k_finalize(const int* list, long long n, const uint8_t* JJ,
+                           const T* L, uint32_t* __restrict__ meta, T* __restrict__ omega,
+                           const int* dn) {
     pdl_wait();
     n = eff_n(dn, n);
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -974,8 +974,8 @@ __global__ void k_finalize(const int* __restrict__ list, long long n, const uint
 
 // Ghost values of one level from coarser active/ghost values (coarse to fine).
 template <typename T>
-__global__ void k_ghost_fill(T* __restrict__ F, const int* __restrict__ glist, long long n, int j, Geom g,
-                             const int* __restrict__ kstop, int jstep) {
+__global__ void k_ghost_fill(T* __restrict__ F, const int* glist, long long n, int j, Geom g,
+                             const int* kstop, int jstep) {
     pdl_wait();
     if (kstop && jstep >= *kstop) return;
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
@@ -986,7 +986,7 @@ __global__ void k_ghost_fill(T* __restrict__ F, const int* __restrict__ glist, l
     pdl_trigger();
 }
 
-__global__ void k_level_counts(const uint32_t* __restrict__ meta, long long n, unsigned long long* counts, Geom g) {
+__global__ void k_level_counts(const uint32_t* meta, long long n, unsigned long long* counts, Geom g) {
     pdl_wait();
     __shared__ unsigned int sc[16];
     if (threadIdx.x < 16) sc[threadIdx.x] = 0;
@@ -1001,7 +1001,7 @@ __global__ void k_level_counts(const uint32_t* __restrict__ meta, long long n, u
     pdl_trigger();
 }
 
-__global__ void k_meta_to_mask(const uint32_t* __restrict__ meta, long long n, uint8_t* __restrict__ mask) {
+__global__ void k_meta_to_mask(const uint32_t* meta, long long n, uint8_t* __restrict__ mask) {
     pdl_wait();
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
          a += (long long)gridDim.x * blockDim.x)
@@ -1009,7 +1009,7 @@ __global__ void k_meta_to_mask(const uint32_t* __restrict__ meta, long long n, u
     pdl_trigger();
 }
 
-__global__ void k_list_to_mask(const int* __restrict__ list, long long n, uint8_t* __restrict__ mask) {
+__global__ void k_list_to_mask(const int* list, long long n, uint8_t* __restrict__ mask) {
     pdl_wait();
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
          a += (long long)gridDim.x * blockDim.x)
@@ -1017,7 +1017,7 @@ __global__ void k_list_to_mask(const int* __restrict__ list, long long n, uint8_
     pdl_trigger();
 }
 
-__global__ void k_meta_unpack(const uint32_t* __restrict__ meta, long long n, int* idx, uint8_t* jx, uint8_t* jy) {
+__global__ void k_meta_unpack(const uint32_t* meta, long long n, int* idx, uint8_t* jx, uint8_t* jy) {
     pdl_wait();
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < n;
          a += (long long)gridDim.x * blockDim.x) {
@@ -1031,8 +1031,8 @@ __global__ void k_meta_unpack(const uint32_t* __restrict__ meta, long long n, in
 
 // Index of every grid point in the combined numbering: active points
 // 0..n_a-1, then the ghosts n_a.. in list order.
-__global__ void k_lat2idx(const int* __restrict__ list, long long n, int* __restrict__ lat2idx,
-                          const int* __restrict__ dcounts, int nkeys) {
+__global__ void k_lat2idx(const int* list, long long n, int* __restrict__ lat2idx,
+                          const int* dcounts, int nkeys) {
     pdl_wait();
     if (dcounts) {
         n = 0;
@@ -1119,9 +1119,9 @@ __constant__ double c_dd4w[4] = {-0.0625, 0.5625, 0.5625, -0.0625};
 __device__ __forceinline__ int row_hash(int key) { return (int)(((unsigned)key * 2654435761u) >> 25); }
 
 __global__ void __launch_bounds__(32 * kRowWarps)
-k_ghost_rows(const int* __restrict__ list, const int* __restrict__ lat2idx, int* __restrict__ row_len,
+k_ghost_rows(const int* list, const int* lat2idx, int* __restrict__ row_len,
              int* __restrict__ row_idx, double* __restrict__ row_w, int rmax, Geom g, int* __restrict__ overflow,
-             const int* __restrict__ dcounts, int nkeys, int* __restrict__ ready, int* __restrict__ err,
+             const int* dcounts, int nkeys, int* __restrict__ ready, int* __restrict__ err,
              unsigned long long limit_ns, int stall) {
     pdl_wait();
     constexpr int kCap = 64;
@@ -1279,9 +1279,9 @@ k_ghost_rows(const int* __restrict__ list, const int* __restrict__ lat2idx, int*
 // predictors' rows read from global memory (no staging).
 template <int P>
 __global__ void __launch_bounds__(32 * kRowWarps)
-k_ghost_rows_wide(const int* __restrict__ list, const int* __restrict__ lat2idx, int* __restrict__ row_len,
+k_ghost_rows_wide(const int* list, const int* lat2idx, int* __restrict__ row_len,
                   int* __restrict__ row_idx, double* __restrict__ row_w, int rmax, Geom g, int* __restrict__ overflow,
-                  const int* __restrict__ dcounts, int nkeys, int* __restrict__ ready, int* __restrict__ err,
+                  const int* dcounts, int nkeys, int* __restrict__ ready, int* __restrict__ err,
                   unsigned long long limit_ns, int stall) {
     pdl_wait();
     constexpr int kCapW = dd_row_max(P);
