@@ -1938,11 +1938,11 @@ wrc_status cfail(BatchCtx& C, wrc_status s, const std::string& msg) {
     } while (0)
 
 // Block plan (krylov_batch_plan): a run gets another block of the launch while
-// its share stays above pt * ept points, the block shape's tile.
+// its share stays above pt * ept points.
 wrc_status plan_batch(BatchCtx& C, const std::vector<wrc_run*>& runs, int& total, int& nitems) {
     const size_t M = runs.size();
     if ((long long)M > krylov_batch_max_runs(C.pt))
-        return cfail(C, WRC_ERR_ARG, "more runs than co-resident blocks of the batched kernel");
+        return cfail(C, WRC_ERR_ARG, "more runs than a batch of this shape takes (8 a SM of shape 64, else 4)");
     std::vector<long long> n(M);
     for (size_t i = 0; i < M; ++i) n[i] = runs[i]->n_active;
     std::vector<int> items, off;

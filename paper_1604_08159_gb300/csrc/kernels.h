@@ -3,6 +3,7 @@
 
 #include <vector>
 
+#include "batch_plan.h"
 #include "common.cuh"
 
 namespace wrc {
@@ -302,11 +303,8 @@ cudaError_t launch_krylov_ex(const KrylovStepArgs& args, const ExArgs& x, const 
 // Batched Krylov step of several problems (device array of arguments) in one
 // cooperative launch of the streaming form: block b works on the items
 // d_off[b] .. d_off[b + 1] - 1, each (problem, block index in it, its
-// blocks).  krylov_batch_plan fills them for problems of n points on sms
-// blocks, a problem getting another block while each keeps `least` points;
-// krylov_batch_max_runs is the most runs a batch of block shape pt accepts.
-void krylov_batch_plan(const std::vector<long long>& n, long long least, int sms, std::vector<int>& items,
-                       std::vector<int>& off);
+// blocks), as krylov_batch_plan (batch_plan.h) fills them;
+// krylov_batch_max_runs is the most runs a batch of shape pt accepts.
 int krylov_batch_max_runs(int pt);
 template <typename T>
 cudaError_t launch_krylov_batch(const KrylovStepArgs* d_args, const int* d_items, const int* d_off, int blocks, int P,

@@ -9,7 +9,6 @@
 #include <algorithm>
 #include <cstdlib>
 #include <mutex>
-#include <numeric>
 
 #include "kernels.h"
 
@@ -336,56 +335,6 @@ int krylov_batch_max_runs(int pt) {
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return -1;
     return sms * (pt == 64 ? 8 : 4);
-}
-
-// Blocks of a batched launch, one per SM.  Up to as many problems as blocks:
-// each gets one, and the rest go one by one to the problem with the most
-// points per block, as long as its share stays above `least` points.  (A
-// launch of 48 mixed members of 9-17K points takes 4.09 ms so, 17 FP64
-// members 1.79, omega and r_v of 65.9K points 1.21; with FP64 dots, 581 and
-// 600 smaller blocks, 5.56, 2.57 and 2.06.)  More problems than blocks: whole problems, the largest first, each to
-// the block with the fewest points so far.
-void krylov_batch_plan(const std::vector<long long>& n, long long least, int sms, std::vector<int>& items,
-                       std::vector<int>& off) {
-    const int M = (int)n.size();
-    items.clear();
-    off.assign(1, 0);
-    if (M <= sms) {
-        std::vector<int> nb(M, 1);
-        for (int used = M; used < sms; ++used) {
-            int best = -1;
-            double most = (double)least;
-            for (int q = 0; q < M; ++q) {
-                const double share = (double)n[q] / nb[q];
-                if (share > most) {
-                    most = share;
-                    best = q;
-                }
-            }
-            if (best < 0) break;
-            nb[best] += 1;
-        }
-        for (int q = 0; q < M; ++q)
-            for (int b = 0; b < nb[q]; ++b) {
-                items.insert(items.end(), {q, b, nb[q]});
-                off.push_back((int)items.size() / 3);
-            }
-        return;
-    }
-    std::vector<int> order(M);
-    std::iota(order.begin(), order.end(), 0);
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
-    std::vector<std::vector<int>> bin(sms);
-    std::vector<long long> load(sms, 0);
-    for (int q : order) {
-        const int b = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-        bin[b].push_back(q);
-        load[b] += n[q];
-    }
-    for (const auto& v : bin) {
-        for (int q : v) items.insert(items.end(), {q, 0, 1});
-        off.push_back((int)items.size() / 3);
-    }
 }
 
 template <typename T>

@@ -8,14 +8,14 @@
 //
 // A problem is worked on by its nb blocks (one block of twelve warps per
 // SM), which meet at its own grid barriers; a problem of one block needs
-// none, and a block may take several of those in turn, so that any number
-// of problems runs in one launch.
+// none.  A block may take several problems in turn (batch_plan.h), so that
+// any number of them runs in one launch.
 //
 // What bounds it: the products' conversions (digits unpacked from 64-bit
 // integers while they are loaded) and their loads, ~300 bytes per point and
 // Arnoldi step at m = 30; the updates follow the scalars of a step, so that
 // each column is read once: its sums, q_j, the next u and its lattice entry.
-// Measured on GB300: see batch_plan() in krylov.cu.
+// Measured on GB300: see krylov_plan() in krylov.cu and batch_plan.h.
 #include "krylov_mma.cuh"
 
 namespace wrc {
@@ -632,8 +632,7 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
 }
 
 // Block b works on items off[b] .. off[b + 1] - 1 in turn: (problem, its
-// block's index in it, its block count); several items only of problems of
-// one block.
+// block's index in it, its block count).
 template <typename T, int P>
 __global__ void __launch_bounds__(kMT, 1) k_krylov_stream(const KrylovStepArgs* __restrict__ args,
                                                           const int* __restrict__ items, const int* __restrict__ off) {

@@ -415,7 +415,7 @@ wrc_status wrc_server_create(const wrc_server_config* cfg, wrc_server** out) {
             g_srv_create_error = "batched Krylov kernel occupancy query failed";
             return WRC_ERR_CUDA;
         }
-        if (cfg->max_slots > lim) return bad("max_slots exceeds the co-resident blocks of the batched kernel");
+        if (cfg->max_slots > lim) return bad("max_slots exceeds the runs a batched launch takes");
     }
     wrc_server* S = new wrc_server();
     S->cfg = *cfg;
