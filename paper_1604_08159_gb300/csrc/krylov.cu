@@ -197,9 +197,19 @@ int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
 
 // Launch rule.  The kernel with its table in shared memory takes every problem
 // that fits one block per SM; beyond, the streaming one.  Points per
-// block: spread over all SMs, but at least 32 (one full warp of the operator;
-// 128^2, 2.7K points: 207 us per launch at 32, 217 at 64, 231 at 128).  The
-// narrow form up to 128 columns (points and ghosts) a block, digits as
+// block: spread over all SMs, but at least 64 (48 at order 8, whose longer
+// ghost rows a block's few warps would queue for), and at order 4 on half of
+// the SMs while that leaves a block at most 128.  A block has its SM to
+// itself, so runs stepped at the same time, each on a stream of its own,
+// share the device only where their blocks leave SMs free; with at least 32
+// points and always all SMs, a run alone was a little faster and several
+// slower than with the FP64 dots (us a step, a run alone and each of eight at
+// once, FP64 dots / 32 points / so: 128^2, 2.8K points 603 / 337 / 345 and
+// 90 / 212 / 82; 256^2, 9.2K points 754 / 445 / 472 and 189 / 297 / 180).
+// Larger problems keep all SMs: alone 1.5 to 1.9 times as fast as with the
+// FP64 dots, four or more at once down to half as fast, where an ensemble's
+// one launch for all is the better form.
+// The narrow form up to 128 columns (points and ghosts) a block, digits as
 // halves while they fit (~370 columns at m = 30), else 64-bit integers
 // (~720): halves and integers measure the same at 220 columns (393 and 394
 // us), the integers being the only form beyond.  Clusters of four blocks,
@@ -207,18 +217,19 @@ int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
 // launches of at most 96 blocks: above, unclustered launches are faster (142
 // blocks: 317 us against 333) and use all SMs.
 // Measured on GB300, one launch, against the kernel with FP64 dots that was
-// used before: 128^2
-// pair, m = 20, 2.7K points 353 -> 207 us; m = 30: 256^2 mixed, 10.8K points
-// 559 -> 317; 1024^2, 17.0K points 483 -> 322; 4096^2 mixed, 28.8K points
-// 752 -> 393; 1024^2, 95.3K points 1321 -> 686; order 2p = 6, 7.4K points
-// 628 -> 370.
+// used before: 128^2 pair, m = 20, 2.8K points 352 -> 219 us; m = 30: 256^2
+// mixed, 10.9K points 553 -> 337; 1024^2, 17.0K points 484 -> 322 and 72.6K
+// 1065 -> 634; 4096^2 mixed, 30.0K points 754 -> 396; order 6, 7.4K points
+// 624 -> 391.
 KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int dev, int cmax) {
     KrylovPlan K;
     const MmaCaps c = caps_of(dev, fp32, P);
     const auto up16 = [](long long x) { return (int)((x + 15) / 16 * 16); };
     {
         int ppb = up16((n + c.cap1 - 1) / std::max(1, c.cap1));
-        if (ppb < 32) ppb = 32;
+        const int half = std::max(1, c.cap1 / 2), wider = up16((n + half - 1) / half);
+        if (P == 2 && wider <= 128) ppb = wider;
+        ppb = std::max(ppb, P == 4 ? 48 : 64);
         int nb = (int)((n + ppb - 1) / ppb);
         nb = nb < 1 ? 1 : nb;
         int cl = 1;
