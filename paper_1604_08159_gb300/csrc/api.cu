@@ -2202,6 +2202,13 @@ void wrc::store_tuned_shape(bool fp32, long long runs, long long active, int pt,
 
 void wrc::mark_batched(wrc_run* R) { R->batched = true; }
 
+// The admission estimate of a run of na points and ng ghosts.  Callers set
+// their budgets by it, so it stays what it was when the basis had the bulk
+// type and each block of a launch three rows of partial sums, although what a
+// run holds (run_device_bytes) has moved: 8 bytes a basis value also in the
+// mixed mode, in batched and streamed launches only, a table of the FP64
+// solve, 17 KB of sums.  It still covers any grid of up to ~0.75 na; a run
+// that holds more is charged what it holds.
 double wrc::run_bytes_for(const wrc_config& cfg, long long na, long long ng) {
     const double N = (double)((long long)cfg.n0 << cfg.J) * (double)((long long)cfg.n0 << cfg.J);
     const double es = cfg.prec == WRC_MIXED ? 4.0 : 8.0;
@@ -2213,15 +2220,13 @@ double wrc::run_bytes_for(const wrc_config& cfg, long long na, long long ng) {
     double b = 7.0 * es * N + 6.0 * N + 8.0 * N + 8.0 * nblk * kMaxKeys + 16.0 * N;
     // FFT tables: twiddles, symbols
     b += 4.0 * es * std::sqrt(N) + 16.0 * std::sqrt(N);
-    if (cfg.prec != WRC_MIXED) b += 4.0 * N + 8.0 * std::sqrt(N);   // the solve's table
     // Krylov small arrays and partial sums (at most kMaxBlocks blocks)
-    b += 8.0 * (m1 * cfg.krylov_m + 33) +
-         8.0 * (double)std::max(krylov_partials_doubles(), (size_t)kMaxBlocks * 4);
+    b += 8.0 * (m1 * cfg.krylov_m + 33) + 8.0 * 3.0 * kMaxBlocks * 66.0;
     const double c = (double)grown_capacity(na), cg = (double)grown_capacity(ng);
     // meta x2, omega x2, details, U, V, g, w, basis (m+1), doubles scratch
-    b += c * (8.0 + 2.0 * es + 5.0 * es + 8.0 * m1 + 8.0);
+    b += c * (8.0 + 2.0 * es + 5.0 * es + es * m1 + 8.0);
     // ghost rows: length, ready flag, dd_row_max(p) indices and weights; ghost basis values
-    b += cg * (8.0 + (4.0 + 8.0) * dd_row_max(cfg.p == 0 ? 2 : cfg.p) + 8.0 * (m1 + 2.0)) + 4.0;
+    b += cg * (8.0 + (4.0 + 8.0) * dd_row_max(cfg.p == 0 ? 2 : cfg.p) + es * m1) + 4.0;
     return b;
 }
 
