@@ -173,8 +173,8 @@ __device__ __noinline__ double scale_slow(double x, int k) { return scalbn(x, k)
 __device__ __noinline__ float scale_slow(float x, int k) { return scalbnf(x, k); }
 __device__ __noinline__ double rsqrt_slow(double q) { return 1.0 / sqrt(q); }
 // FP32 value of a double rounded towards zero, by integer operations (the
-// conversion instruction takes an FP64 issue slot); for |x| in [2^-100, 2^100],
-// else 0 or the largest.
+// conversion instruction takes an FP64 issue slot); |x| below 2^100, 0 below
+// 2^-100.
 __device__ __forceinline__ float d2f_trunc(double x) {
     const int hi = __double2hiint(x), e = (hi >> 20) & 0x7ff;
     const unsigned f = ((unsigned)(e - 1023 + 127) << 23) | ((unsigned)(hi & 0xfffff) << 3) |
@@ -1196,7 +1196,9 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                 const int euu = __shfl_sync(0xffffffffu, expo(val), j & 31) - 1023;
                 s_fs[lane] = lane < j ? d2f_trunc(scale2(val, 1022 - e)) : 0.f;
                 const int gap = j == 0 || e == 0 ? 1000 : euu - 2 * (e - 1022);
-                if (lane == 0) s_int[1] = gap >= 64 ? 3 : gap >= 32 ? 2 : gap >= 24 ? 1 : 0;
+                // (3 has H in FP32: its largest entries are near |A|, which must be mid-range)
+                const bool mid = eA >= -60 && eA <= 90;
+                if (lane == 0) s_int[1] = gap >= 64 && mid ? 3 : gap >= 32 ? 2 : gap >= 24 ? 1 : 0;
             }
         } else if (wid == 8) {
             if (lane < 3) s_e[lane] = 0;
