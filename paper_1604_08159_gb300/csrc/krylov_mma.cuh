@@ -3,8 +3,8 @@
 // cooperative kernel whose orthogonalisation runs on the tensor cores.
 //
 // Method: that of krylov_impl.cuh -- Arnoldi with classical Gram-Schmidt
-// applied twice, the second pass delayed by one step -- with b itself taken
-// as the first "u": step j applies A to u (z = A u), one reduction gives
+// applied twice, the second pass delayed by one step -- with b itself (times
+// a power of two, first_scale) taken as the first "u": step j applies A to u (z = A u), one reduction gives
 // s = Q^T u, |u|^2, t = Q^T z and u.z, and
 //   q_j = (u - Q s) / h,  h^2 = |u|^2 - |s|^2  (step 0: h = beta, q_0 = b / beta),
 //   next u = (z - Q t - q_j qz) / h,  qz = (u.z - s.t) / h.
@@ -261,6 +261,15 @@ __device__ __forceinline__ double scale2(double x, int k) {
         return __hiloint2double(__double2hiint(x) + (k << 20), __double2loint(x));
     if (__double_as_longlong(x) << 1 == 0) return x;
     return scale_slow(x, k);
+}
+// The exponent by which a first vector b of largest magnitude below 2^(e - 1022)
+// (e biased) is scaled: with b itself as the first u, z = A u, in the bulk
+// type, has the scale of |b| |A| and u.z that of |b|^2 |A|; 0 (mid-range) in
+// all but unusual units.
+template <typename T>
+__device__ __forceinline__ int first_scale(int e) {
+    const int E = e - 1022;
+    return e == 0 || e == 0x7ff || abs(E) <= (sizeof(T) == 4 ? 30 : 200) ? 0 : E;
 }
 // 2^k as a double, 0 below the normal range.
 __device__ __forceinline__ double pow2d(int k) {
@@ -953,6 +962,19 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
         atomicMax(&slot[4], (unsigned)s_e[6]);
     }
     if (!meet()) return calls;
+    const int be = first_scale<T>((int)__ldcg(&slot[0]));   // the same for every block
+    if (be != 0) {   // u = b 2^-be
+        for (int c = threadIdx.x; c < Y.cols; c += kMT) {
+            const bool gh = c >= ppb;
+            if (gh ? c - ppb >= ng : c >= n) continue;
+            const int gp = gh ? gpos[c - ppb] : 0;
+            const T v = (T)scale2(us[c], -be);
+            us[c] = dbl(v);
+            lattice(gh ? (gp >> 29) & 3 : field(p0 + c))[gh ? gp & 0xffffff : meta_pos(meta[c])] = v;
+        }
+        if (threadIdx.x < 2 && s_e[threadIdx.x]) s_e[threadIdx.x] = max(0, s_e[threadIdx.x] - be);
+        if (!meet()) return calls;
+    }
 
     const int nunit = (n + 15) / 16;
     const int nact = min(kPW, nunit);                    // product warps with points
@@ -978,7 +1000,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
         }
         // ---- z = A u at the own points ------------------------------------
         if (wid == 8) {
-            if (lane == 0) s_e[3] = (int)__ldcg(&slot[(j & 1) * 2]);
+            if (lane == 0) s_e[3] = (int)__ldcg(&slot[(j & 1) * 2]) - (j == 0 ? be : 0);
             // the other parity's sums and exponents (last read before the barrier just passed)
             for (int q = bid; q < kCopies; q += nb) {
                 unsigned long long* z = acc + (((j + 1) & 1) * kCopies + q) * 128;
@@ -1315,7 +1337,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
         __syncthreads();
         const int stop = s_int[0];
         if (j == 0 && threadIdx.x == 0) {
-            const double b = s_sc[0] > 0.0 && finite_bits(s_sc[0]) ? s_sc[0] * s_sc[1] : s_sc[0];
+            const double b = scale2(s_sc[0] > 0.0 && finite_bits(s_sc[0]) ? s_sc[0] * s_sc[1] : s_sc[0], be);
             s_sc[3] = b;
             if (lead) *A.beta = b;
         }

@@ -186,6 +186,22 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
         atomicMax(&slot[4], (unsigned)s_e[6]);
     }
     if (!meet()) return;
+    const int be = first_scale<T>(solo ? s_e[1] : (int)__ldcg(&slot[0]));
+    if (be != 0) {   // as in krylov_mma_body
+        for (int c = threadIdx.x; c < n; c += kMT) {
+            const T v = (T)scale2(dbl(us[c]), -be);
+            us[c] = v;
+            Lq[meta_pos(meta[c])] = v;
+        }
+        for (int c = threadIdx.x; c < ng; c += kMT) {
+            const T v = (T)scale2(ug[c], -be);
+            ug[c] = dbl(v);
+            Lq[A.glist[t0 + c]] = v;
+        }
+        __syncthreads();   // s_e[1] has been read
+        if (threadIdx.x < 2 && s_e[threadIdx.x]) s_e[threadIdx.x] = max(0, s_e[threadIdx.x] - be);
+        if (!meet()) return;
+    }
 
     const int nunit = (n + 15) / 16;
     const int nact = min(kSW, nunit);
@@ -196,7 +212,7 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
         unsigned long long* accj = acc + (j & 1) * kCopies * 128;
         // ---- column j - 1 of H (warp 8), z = A u at the own points ------------
         if (wid == 8) {
-            if (lane == 0) s_e[3] = solo ? s_e[1] : (int)__ldcg(&slot[(j & 1) * 2]);
+            if (lane == 0) s_e[3] = solo ? s_e[1] : (int)__ldcg(&slot[(j & 1) * 2]) - (j == 0 ? be : 0);
             for (int q = bid; q < kCopies && !solo; q += nb) {
                 unsigned long long* z = acc + (((j + 1) & 1) * kCopies + q) * 128;
                 for (int t = lane; t < 128; t += 32) z[t] = 0ull;
@@ -479,7 +495,7 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
         if (threadIdx.x == 0) {
             s_next = 0;
             if (j == 0) {
-                const double b = s_sc[0] > 0.0 && finite_bits(s_sc[0]) ? s_sc[0] * s_sc[1] : s_sc[0];
+                const double b = scale2(s_sc[0] > 0.0 && finite_bits(s_sc[0]) ? s_sc[0] * s_sc[1] : s_sc[0], be);
                 s_sc[3] = b;
                 if (lead) *A.beta = b;
             }
