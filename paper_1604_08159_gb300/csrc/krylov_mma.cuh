@@ -535,7 +535,8 @@ __device__ __forceinline__ T op_apply(const T* F, const OpPoint<T>& c, T r, cons
     }
 }
 
-// Absolute sum of the operator's row at a point: |A q| <= it times max |q|.
+// Absolute sum of the operator's row, without the friction r, at a point:
+// |(A + r) q| <= it times max |q|.
 template <typename T, int P>
 __device__ __forceinline__ double row_bound(const KrylovStepArgs& A, uint32_t mw, T U, T V) {
     double d1 = 0.0, d2 = -dd_d2(P, 0);
@@ -545,7 +546,7 @@ __device__ __forceinline__ double row_bound(const KrylovStepArgs& A, uint32_t mw
     for (int o = 1; o <= P; ++o) d2 += 2.0 * (dd_d2(P, o) < 0 ? -dd_d2(P, o) : dd_d2(P, o));
     const int shx = A.g.J - meta_jx(mw), shy = A.g.J - meta_jy(mw);
     return d1 * (fabs(dbl(U)) * pow2_down(A.c1J, shx) + fabs(dbl(V)) * pow2_down(A.c1J, shy)) +
-           d2 * A.nu * (pow2_down(A.c2J, 2 * shx) + pow2_down(A.c2J, 2 * shy)) + fabs(A.r);
+           d2 * A.nu * (pow2_down(A.c2J, 2 * shx) + pow2_down(A.c2J, 2 * shy));
 }
 // Extra scale bits of a ghost's basis values: its interpolation row's
 // absolute sum beyond 1.9, as powers of two (basis values hold up to 2).
@@ -839,6 +840,12 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
     T* Lq = (T*)A.Lq;
     T* zb = (T*)A.w;                   // z at every active point (read by the ghosts' rows)
     const T nu = (T)A.nu, r = (T)A.r, c1J = (T)A.c1J, c2J = (T)A.c2J;
+    // The steps apply A + r I: the same vectors, H + r I.  The ghost values of u
+    // follow from those of z by the points' recurrence, which carries a
+    // rounding d_0 of theirs on as d_{j+1} = -sum_q H_qj d_q / h_{j+1}: with H
+    // near -r I it grew by r / h a step (r = 50: 10 to 100), until the ghost
+    // values left the range of their fixed point.
+    const bool shift = !EX && A.r != 0.0;
     // field and point of stacked entry e, field and ghost of stacked ghost t; a field's lattice
     const int xn = EX ? X->n : 0, xg = EX ? X->ng : 0;
     const auto field = [&](long long e) { return EX ? (e >= 2LL * xn ? 2 : (e >= xn ? 1 : 0)) : 0; };
@@ -1043,7 +1050,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                     sH[lane * 33 + q] = v;
                     if (nrc >= 0) sHf[lane * 33 + q] = d2f_trunc(v);
                 }
-                const int ev = (int)__reduce_max_sync(0xffffffffu, (unsigned)expo(v));
+                const int ev = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(expo(v), shift ? expo(A.r) : 0));
                 if (lane == 0) s_e[7] = ev;
             }
         } else if (!last) {
@@ -1056,11 +1063,11 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                         const int f = field(p0 + p);
                         z = (T)ex_entry<P>(*X, meta[p], f, (int)(p0 + p - (long long)f * xn));
                     } else if (c == opw * 32) {
-                        z = op_apply<T, P>(Lq, op0, r, A.g, c1J, c2J);
+                        z = op_apply<T, P>(Lq, op0, T(0), A.g, c1J, c2J);
                     } else {
                         OpPoint<T> op;
                         op_prepare<T, P>(op, meta[p], Ua[p], Va[p], nu, A.g, c1J, c2J);
-                        z = op_apply<T, P>(Lq, op, r, A.g, c1J, c2J);
+                        z = op_apply<T, P>(Lq, op, T(0), A.g, c1J, c2J);
                     }
                     zb[p0 + p] = z;
                     const double zd = dbl(z);
@@ -1218,7 +1225,7 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                 const int euu = __shfl_sync(0xffffffffu, expo(val), j & 31) - 1023;
                 s_fs[lane] = lane < j ? d2f_trunc(scale2(val, 1022 - e)) : 0.f;
                 const int gap = j == 0 || e == 0 ? 1000 : euu - 2 * (e - 1022);
-                // (3 has H in FP32: its largest entries are near |A|, which must be mid-range)
+                // (3 has H in FP32: its largest entries are near |A + r I|, which must be mid-range)
                 const bool mid = eA >= -60 && eA <= 90;
                 if (lane == 0) s_int[1] = gap >= 64 && mid ? 3 : gap >= 32 ? 2 : gap >= 24 ? 1 : 0;
             }
@@ -1273,7 +1280,8 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
                 if (expo(q2) == 0 || expo(q2) - 1023 <= em) {
                     double thr = 0.0;
                     if (j > 0) {
-                        const double hv = in ? sH[lane * 33 + j - 1] : 0.0;
+                        double hv = in ? sH[lane * 33 + j - 1] : 0.0;
+                        if (shift && lane == j - 1) hv -= A.r;
                         double hh = hv * hv;
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
@@ -1401,6 +1409,8 @@ __device__ __forceinline__ int krylov_mma_body(const KrylovStepArgs& A, const in
     if (wid == 8 && k > 0) {
         if (lane < k) sH[lane * 33 + k - 1] += s_v[0][lane];
         if (lane == 0) sH[k * 33 + k - 1] = s_sc[0] > 0.0 && finite_bits(s_sc[0]) ? s_sc[0] * s_sc[1] : s_sc[0];
+        __syncwarp();
+        if (shift && lane < k) sH[lane * 33 + lane] -= A.r;   // H of A
     }
     __syncthreads();
     if (bid == 0)

@@ -101,6 +101,7 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
     double* rz = ug + ldg;
     int* gsx = (int*)((double*)A.Gb + (size_t)(m + 2) * ldg) + t0;
     const T nu = (T)A.nu, r = (T)A.r, c1J = (T)A.c1J, c2J = (T)A.c2J;
+    const bool shift = A.r != 0.0;       // the steps apply A + r I, as in krylov_mma_body
     unsigned long long* acc = reinterpret_cast<unsigned long long*>(A.part);
     unsigned* slot = reinterpret_cast<unsigned*>(acc + 2 * kCopies * 128);
     const bool solo = nb == 1;           // no other block: no grid barrier
@@ -232,7 +233,7 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
                 if (lane < q) v = (s_v[1][lane] - gi) * hinv;
                 else if (lane == q) v = (qz - (q > 0 ? h * s_v[0][q - 1] : 0.0)) * hinv;
                 if (lane <= q) sH[lane * 33 + q] = v;
-                const int ev = (int)__reduce_max_sync(0xffffffffu, (unsigned)expo(v));
+                const int ev = (int)__reduce_max_sync(0xffffffffu, (unsigned)max(expo(v), shift ? expo(A.r) : 0));
                 if (lane == 0) s_e[7] = ev;
             }
         }
@@ -258,7 +259,7 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
                 fetch(c + 64 * kSW);
                 T z[2];
 #pragma unroll
-                for (int q = 0; q < 2; ++q) z[q] = op_apply<T, P>(Lq, op[q], r, A.g, c1J, c2J);
+                for (int q = 0; q < 2; ++q) z[q] = op_apply<T, P>(Lq, op[q], T(0), A.g, c1J, c2J);
                 int e = 0;
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
@@ -446,7 +447,8 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
             if (stop == 0) {
                 double thr = 0.0;
                 if (j > 0) {
-                    const double hv = in ? sH[lane * 33 + j - 1] : 0.0;
+                    double hv = in ? sH[lane * 33 + j - 1] : 0.0;
+                    if (shift && lane == j - 1) hv -= A.r;
                     double hh = hv * hv;
 #pragma unroll
                     for (int o = 16; o > 0; o >>= 1) hh += __shfl_xor_sync(0xffffffffu, hh, o);
@@ -596,6 +598,8 @@ __device__ __forceinline__ void krylov_stream_body(const KrylovStepArgs& A, cons
     if (wid == 8 && k > 0) {
         if (lane < k) sH[lane * 33 + k - 1] += s_v[0][lane];
         if (lane == 0) sH[k * 33 + k - 1] = s_sc[0] > 0.0 && finite_bits(s_sc[0]) ? s_sc[0] * s_sc[1] : s_sc[0];
+        __syncwarp();
+        if (shift && lane < k) sH[lane * 33 + lane] -= A.r;   // H of A
     }
     __syncthreads();
     if (bid == 0)
