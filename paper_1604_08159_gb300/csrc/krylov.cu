@@ -197,18 +197,19 @@ int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
 
 // Launch rule.  The kernel with its table in shared memory takes every problem
 // that fits one block per SM; beyond, the streaming one.  Points per
-// block: spread over all SMs, but at least 64 (48 at order 8, whose longer
-// ghost rows a block's few warps would queue for), and at order 4 on half of
-// the SMs while that leaves a block at most 128.  A block has its SM to
-// itself, so runs stepped at the same time, each on a stream of its own,
-// share the device only where their blocks leave SMs free; with at least 32
-// points and always all SMs, a run alone was a little faster and several
-// slower than with the FP64 dots (us a step, a run alone and each of eight at
-// once, FP64 dots / 32 points / so: 128^2, 2.8K points 603 / 337 / 345 and
-// 90 / 212 / 82; 256^2, 9.2K points 754 / 445 / 472 and 189 / 297 / 180).
-// Larger problems keep all SMs: alone 1.5 to 1.9 times as fast as with the
-// FP64 dots, four or more at once down to half as fast, where an ensemble's
-// one launch for all is the better form.
+// block: spread over all SMs, but at least 48 at order 4 and 32 above (the
+// higher orders' longer ghost rows queue for a block's few warps: 64 points
+// make a mixed run of 3-4K points 8-10% slower).  A block has its SM to itself, so
+// runs stepped at the same time, each on a stream of its own, share the
+// device only where their blocks leave SMs free.  48 points cost a run alone
+// nothing and let two small ones run side by side (128^2, 2.8K points, us a
+// step alone / each of four / each of eight at once: 603 / 166 / 90 with the
+// FP64 dots, 337 / 213 / 212 from 32 points on, 335 / 115 / 112 from 48, 345
+// / 100 / 82 from 64).  Larger runs keep all SMs, as half of them cost a run
+// alone 3-10% (256^2, 9.2K points: 754 / 241 / 189, 445 / 294 / 297, on half
+// the SMs 472 / 181 / 180): alone they take 0.5 to 0.7 of the time with the
+// FP64 dots, four or eight at once up to 1.9 times it; an ensemble's one
+// launch for all its members is the form for many.
 // The narrow form up to 128 columns (points and ghosts) a block, digits as
 // halves while they fit (~370 columns at m = 30), else 64-bit integers
 // (~720): halves and integers measure the same at 220 columns (393 and 394
@@ -217,7 +218,7 @@ int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
 // launches of at most 96 blocks: above, unclustered launches are faster (142
 // blocks: 317 us against 333) and use all SMs.
 // Measured on GB300, one launch, against the kernel with FP64 dots that was
-// used before: 128^2 pair, m = 20, 2.8K points 352 -> 219 us; m = 30: 256^2
+// used before: 128^2 pair, m = 20, 2.8K points 352 -> 209 us; m = 30: 256^2
 // mixed, 10.9K points 553 -> 337; 1024^2, 17.0K points 484 -> 322 and 72.6K
 // 1065 -> 634; 4096^2 mixed, 30.0K points 754 -> 396; order 6, 7.4K points
 // 624 -> 391.
@@ -227,9 +228,7 @@ KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int d
     const auto up16 = [](long long x) { return (int)((x + 15) / 16 * 16); };
     {
         int ppb = up16((n + c.cap1 - 1) / std::max(1, c.cap1));
-        const int half = std::max(1, c.cap1 / 2), wider = up16((n + half - 1) / half);
-        if (P == 2 && wider <= 128) ppb = wider;
-        ppb = std::max(ppb, P == 4 ? 48 : 64);
+        ppb = std::max(ppb, P == 2 ? 48 : 32);
         int nb = (int)((n + ppb - 1) / ppb);
         nb = nb < 1 ? 1 : nb;
         int cl = 1;

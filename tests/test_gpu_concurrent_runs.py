@@ -1,7 +1,7 @@
 """Independent runs stepped by a thread and on a stream each: the results of a
 run alone, bit for bit, and small runs share the device -- eight at once have
-at least 2.5 times the throughput of one (with launches over most of the SMs
-they had 1.6 times, with half as many blocks 4)."""
+at least 2.2 times the throughput of one (with launches over most of the SMs
+they had 1.6 times, with blocks of 48 points 3)."""
 
 import threading
 import time
@@ -62,7 +62,7 @@ def test_eight_small_runs(prec):
         for r in runs:
             for got, want in zip(r.active(), alone):
                 assert np.array_equal(got, want)
-        assert 8 * one / all8 >= 2.5, (one, all8)
+        assert 8 * one / all8 >= 2.2, (one, all8)
     finally:
         for r in runs:
             r.close()
