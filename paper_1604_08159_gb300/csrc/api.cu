@@ -10,6 +10,7 @@
 #include <mutex>
 #include <tuple>
 #include <cstdio>
+#include <cstdlib>
 #include <vector>
 #include <cstring>
 #include <string>
@@ -216,6 +217,7 @@ struct wrc_run {
     // lattices of a Krylov vector's v and pi parts (Lq its u part), xd the
     // state's derivatives at the active points (8 x cap)
     bool exner = false;
+    bool ex_even = false;    // its fields' parts of a Krylov vector have scales within 2^12 (exner_threshold_whole)
     DevBuf pe[2], Lp, Lqx, xd, xbasis, xw;
 };
 
@@ -1019,7 +1021,7 @@ wrc_status exner_krylov(wrc_run* R) {
     CK(ex_scatter_fields(a, fs, Lb, nullptr, 0, s));
     CK(ex_base(a, K.w, s));
     const KrylovPlan plan = krylov_ex_plan(n, R->n_ghost, m, R->g.P, R->device);
-    if (plan.form < 3) {
+    if (plan.form < 3 && R->ex_even) {
         KrylovStepArgs A{};
         A.g = R->g;
         A.meta = a.meta;
@@ -1163,10 +1165,31 @@ wrc_status init_field_t(wrc_run* R, const double* omega_lattice, int device_ptr)
 
 // Velocity-Exner initial condition: u, v, pi on the whole lattice in L, Lr,
 // Lp; the joint thresholding of their full-lattice transforms.
+// Also whether the step's Krylov vectors may be held to one absolute
+// precision: A takes a velocity q to pi div q and q . grad pi, and a pi q to
+// C grad q, beside advection and sound at a speed w, so that beside a larger
+// part of scale 1 the other has pi / w or C / w at least.  A part below 2^-12
+// keeps fewer than 49 of the basis values' 61 bits: such a run takes the kernel
+// with FP64 dots (with C = 3e5, pi = 1, as in SI units, the ratios are
+// 2^-9.1 and 2^9.1).
 wrc_status exner_threshold_whole(wrc_run* R) {
+    CK(cudaMemsetAsync(R->flag_dev + 2, 0, 2 * sizeof(int), R->st));
+    CK(ex_scales((const double*)R->L, R->Lr.as<double>(), R->Lp.as<double>(), R->N, R->flag_dev + 2, R->st));
+    int* const hi = R->counts_host + kMaxKeys + 2;   // read after the wait in rebuild_host
+    CK(cudaMemcpyAsync(hi, R->flag_dev + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, R->st));
     CK(cudaMemsetAsync(R->act, 1, R->N, R->st));
     R->n_active = 0;
-    return threshold_current<double>(R, R->cfg.eps, true);
+    TRY(threshold_current<double>(R, R->cfg.eps, true));
+    const auto value = [](int h) {
+        const uint64_t b = (uint64_t)(uint32_t)h << 32;
+        double x;
+        std::memcpy(&x, &b, sizeof x);
+        return x;
+    };
+    const double C = R->cfg.cpt, pi = value(hi[1]);
+    const double w = std::max({value(hi[0]), std::fabs(R->cfg.gx), std::fabs(R->cfg.gy), std::sqrt(C * pi)});
+    R->ex_even = std::min(C, pi) >= w / 4096.0 && w > 0.0 && std::isfinite(w);
+    return WRC_OK;
 }
 
 template <typename T>

@@ -10,6 +10,8 @@
 // active points, the ghosts through the interpolation rows), the operator
 // and classical Gram-Schmidt twice -- krylov_mma.cuh's while its table fits
 // the SMs' shared memory, else k_ex_krylov here.  No Poisson solve.
+#include <algorithm>
+
 #include "exner_op.cuh"
 #include "krylov_impl.cuh"
 #include "wrc.h"
@@ -399,6 +401,23 @@ __global__ void __launch_bounds__(kExKrylovThreads, 1) k_ex_krylov(ExArgs a, ExK
     }
 }
 
+// The largest magnitudes of the velocity (out[0]) and of pi (out[1]) on the
+// lattice, as the high words of the doubles (out zeroed by the caller).
+__global__ void k_ex_scales(const double* __restrict__ u, const double* __restrict__ v, const double* __restrict__ pi,
+                            long long n, int* __restrict__ out) {
+    int a = 0, b = 0;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+        a = max(a, max(__double2hiint(u[e]) & 0x7fffffff, __double2hiint(v[e]) & 0x7fffffff));
+        b = max(b, __double2hiint(pi[e]) & 0x7fffffff);
+    }
+    a = (int)__reduce_max_sync(0xffffffffu, (unsigned)a);
+    b = (int)__reduce_max_sync(0xffffffffu, (unsigned)b);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, a);
+        atomicMax(out + 1, b);
+    }
+}
+
 __global__ void k_ex_fill(double* __restrict__ F, long long n, double value) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         F[i] = value;
@@ -448,6 +467,12 @@ cudaError_t ex_krylov(const ExArgs& a, const ExKrylov& K, int blocks, cudaStream
                                         0, s);
     });
     if (e != cudaSuccess) return e;
+    note_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t ex_scales(const double* u, const double* v, const double* pi, long long n, int* out, cudaStream_t s) {
+    k_ex_scales<<<std::min(ex_blocks(n), 608), kExThreads, 0, s>>>(u, v, pi, n, out);
     note_launch();
     return cudaGetLastError();
 }

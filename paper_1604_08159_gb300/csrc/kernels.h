@@ -195,6 +195,9 @@ cudaError_t ex_scatter_fields(const ExArgs& a, const double* const src[3], doubl
 // First derivatives and Laplacians of the state at the active points (into
 // a.d) and the right-hand side F(U^n) stacked into w (3 n).
 cudaError_t ex_base(const ExArgs& a, double* w, cudaStream_t s);
+// Largest magnitudes of velocity and pi on the lattices, as high words of
+// doubles, into out[0] and out[1] (zeroed by the caller).
+cudaError_t ex_scales(const double* u, const double* v, const double* pi, long long n, int* out, cudaStream_t s);
 // Fill a lattice with a constant.
 cudaError_t ex_fill(double* F, long long n, double value, cudaStream_t s);
 // The whole Krylov projection of a velocity-Exner step too large for
