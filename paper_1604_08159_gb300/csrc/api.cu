@@ -37,6 +37,14 @@ void wrc::note_launch() {
 }
 long long wrc::launches_total() { return g_launches.load(std::memory_order_relaxed); }
 
+cudaError_t wrc::device_malloc(void** p, size_t bytes) {
+    const char* lim = std::getenv("WRC_ALLOC_TEST_LIMIT");
+    const cudaError_t e =
+        lim && bytes > std::strtoull(lim, nullptr, 10) ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    if (e != cudaSuccess) cudaGetLastError();   // reported by the caller, not by the next launch's check
+    return e;
+}
+
 namespace {
 
 // Happy breakdown of the Arnoldi process: h_{j+1,j} <= tol |A v_j|.
@@ -54,13 +62,8 @@ struct DevBuf {
     cudaError_t grow(size_t need, size_t keep, cudaStream_t s) {
         if (need <= bytes) return cudaSuccess;
         void* q = nullptr;
-        // test switch: a growth beyond so many bytes fails as if the device were full
-        const char* lim = std::getenv("WRC_ALLOC_TEST_LIMIT");
-        cudaError_t e = lim && need > std::strtoull(lim, nullptr, 10) ? cudaErrorMemoryAllocation : cudaMalloc(&q, need);
-        if (e != cudaSuccess) {
-            cudaGetLastError();   // reported by the caller, not by the next launch's check
-            return e;
-        }
+        cudaError_t e = device_malloc(&q, need);
+        if (e != cudaSuccess) return e;
         if (p && keep) {
             e = cudaMemcpyAsync(q, p, keep, cudaMemcpyDeviceToDevice, s);
             if (e != cudaSuccess) return e;
@@ -1413,7 +1416,7 @@ wrc_status wrc_create(const wrc_config* cfg, void* cuda_stream, wrc_run** out) {
     const long long N = R->N;
     const int m = cfg->krylov_m;
     const int nblk = (int)((N + kTile - 1) / kTile);
-    auto alloc = [&](void** p, size_t bytes) { return cudaMalloc(p, bytes); };
+    auto alloc = [&](void** p, size_t bytes) { return device_malloc(p, bytes); };
     cudaError_t e = cudaSuccess;
     void** lp[] = {(void**)&R->L, (void**)&R->Lq, (void**)&R->psi};
     for (auto p : lp)
@@ -1475,10 +1478,10 @@ wrc_status wrc_create(const wrc_config* cfg, void* cuda_stream, wrc_run** out) {
             return ex == cudaErrorMemoryAllocation ? WRC_ERR_OOM : WRC_ERR_CUDA;
         }
     }
-    if (poisson_plan_init(R->plan, R->g, R->fp32, R->st) != 0) {
-        g_create_error = "FFT/expm kernel set-up failed";
+    if (const int pe = poisson_plan_init(R->plan, R->g, R->fp32, R->st); pe != 0) {
+        g_create_error = pe == -1 ? "allocation failed: tables of the streamfunction solve" : "FFT/expm kernel set-up failed";
         free_run(R);
-        return WRC_ERR_CUDA;
+        return pe == -1 ? WRC_ERR_OOM : WRC_ERR_CUDA;
     }
     if (cudaStreamSynchronize(R->st) != cudaSuccess) {
         g_create_error = std::string("set-up: ") + cudaGetErrorString(cudaGetLastError());

@@ -717,16 +717,16 @@ int setup_all() {
 
 template <typename T>
 int plan_init_t(PoissonPlan& p, const Geom& g, cudaStream_t s) {
-    if (cudaMalloc(&p.tw, sizeof(cx_t<T>) * p.n) != cudaSuccess) return -1;
-    if (cudaMalloc(&p.ptw, sizeof(cx_t<T>) * 2 * p.n) != cudaSuccess) return -1;
-    if (cudaMalloc(&p.sigma, sizeof(T) * p.n) != cudaSuccess) return -1;
-    if (cudaMalloc(&p.dsym, sizeof(T) * p.n) != cudaSuccess) return -1;
+    if (device_malloc(&p.tw, sizeof(cx_t<T>) * p.n) != cudaSuccess) return -1;
+    if (device_malloc(&p.ptw, sizeof(cx_t<T>) * 2 * p.n) != cudaSuccess) return -1;
+    if (device_malloc(&p.sigma, sizeof(T) * p.n) != cudaSuccess) return -1;
+    if (device_malloc(&p.dsym, sizeof(T) * p.n) != cudaSuccess) return -1;
     if (setup_all<T>() != 0) return -2;
     { launch_pdl(k_fft_init<T>, (p.n + 255) / 256, 256, 0, s, (cx_t<T>*)p.tw, (T*)p.sigma, (T*)p.dsym, p.n,
                                                        g.h, g.P); note_launch(); }
     if constexpr (std::is_same<T, double>::value) {
         const size_t N = (size_t)(p.n / 2 + 1) * p.n;
-        if (cudaMalloc(&p.inv, sizeof(double) * N) != cudaSuccess) return -1;
+        if (device_malloc(&p.inv, sizeof(double) * N) != cudaSuccess) return -1;
         k_fx_pass_tables<<<(p.n + 255) / 256, 256, 0, s>>>((int4*)p.ptw, p.n, p.logn, fx_log_e(p.logn));
         k_fx_symbol<<<blocks_for((long long)N), kThreads, 0, s>>>((double*)p.inv, (const double*)p.sigma, p.n);
         note_launch();

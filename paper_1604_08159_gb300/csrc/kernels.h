@@ -8,6 +8,10 @@
 
 namespace wrc {
 
+// cudaMalloc whose failure leaves no pending error behind; sizes beyond the
+// test switch WRC_ALLOC_TEST_LIMIT (bytes) fail as if the device were full.
+cudaError_t device_malloc(void** p, size_t bytes);
+
 // ---- grid.cu: lattice, transform, thresholding, index sets -----------------
 template <typename T>
 void launch_init_vortices(T* L, const double* params, int n, const Geom& g, cudaStream_t s);
@@ -71,6 +75,7 @@ struct PoissonPlan {
     void* dsym = nullptr;    // symbol of the 4th-order first-derivative stencil (imaginary part)
     void* inv = nullptr;     // FP64: 1/(n^2 (sigma(kx) + sigma(ky))), kx <= n/2 (see fft_fixed.cuh)
 };
+// 0, or -1 where the device memory for its tables cannot be had, or below.
 int poisson_plan_init(PoissonPlan& p, const Geom& g, bool fp32, cudaStream_t s);
 void poisson_plan_free(PoissonPlan& p);
 // psi = L_h^{-1}(-(R - mean R)), mean(psi) = 0; C1, C2 are NJ*NJ complex work

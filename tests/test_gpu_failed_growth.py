@@ -79,3 +79,19 @@ def test_rosenbrock_run(monkeypatch):
         run.step(1)
         for got, want in zip(run.active(), ref):
             assert np.array_equal(got, want)
+
+
+def test_tables_of_the_solve(monkeypatch):
+    """The FP64 solve's table, the largest of a run's tables: a failed
+    allocation of it is out of memory (a server waits and tries again), and
+    leaves nothing pending."""
+    prm = small_params(n0=32, J=4)   # (n / 2 + 1) n doubles: 1.05 MB
+    monkeypatch.setenv("WRC_ALLOC_TEST_LIMIT", str(1 << 20))
+    with pytest.raises(B.WrcError) as e:
+        B.Run(prm)
+    assert e.value.status == -2
+    monkeypatch.delenv("WRC_ALLOC_TEST_LIMIT")
+    with B.Run(prm) as run:
+        run.init_vortices(VORT)
+        run.step(1)
+        run.sync()
