@@ -291,14 +291,10 @@ wrc_status wrc_query_stages(wrc_run* run, double* out, int32_t cap);
  * mode 2): for each grid barrier p it passed, out[4p..4p+3] = the first and
  * the last arrival of its blocks, the index of the last block to arrive, and
  * the release of block 0, in microseconds from the start of block 0 (device
- * global timer).  In the tensor-core kernel (every problem whose basis fits
- * the shared memory of the co-resident blocks) barrier 0 follows
- * b = A_n omega + g, barrier 1 the ghost values of b; then each Arnoldi step
- * has two: after its dots and after the new vectors (the last step stops
- * after its dots; phi_1 and the update follow without a barrier).  In the
- * FP64 kernel barrier 1 follows the ghost values of v_0, barriers 2 and 3
- * the first projection of A v_0, each further step has two, and the final
- * barrier follows phi_1, before the update.
+ * global timer).  Barrier 0 follows b = A_n omega + g, barrier 1 the ghost
+ * values of b (one more where b is far from 1 and is scaled); then each
+ * Arnoldi step has two: after its dots and after the new vectors (the last
+ * step stops after its dots; phi_1 and the update follow without a barrier).
  * *nphases receives the count.  WRC_ERR_ARG if cap < 4 * count; WRC_ERR_STATE without a traced
  * launch.  Synchronises. */
 wrc_status wrc_query_phase_trace(wrc_run* run, double* out, int32_t cap, int32_t* nphases);

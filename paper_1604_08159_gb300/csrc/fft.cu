@@ -582,13 +582,14 @@ __global__ void k_transpose(const C* in, C* __restrict__ out, int rows, int cols
 //           n_0 = -2 sum n_j, sigma = 4 sum_j n_j sin^2(j theta/2)/(d2 h^2)
 //           (no cancellation at small theta), and with the first-derivative
 //           stencil (n_1..n_R)/(d1 h), d = 2 sum_j n_j sin(j theta)/(d1 h).
+// tw and dsym may be null (an FP64 run has no use for them).
 template <typename T>
 __global__ void k_fft_init(cx_t<T>* tw, T* sigma, T* dsym, int n, double h, int P) {
     pdl_wait();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
         double sn, cs;
         sincospi(2.0 * t / n, &sn, &cs);
-        tw[t] = mk<cx_t<T>>((T)cs, (T)(-sn));
+        if (tw) tw[t] = mk<cx_t<T>>((T)cs, (T)(-sn));
         if (P == 3 || P == 4) {
             double sg = 0.0, ds = 0.0;
             for (int j = 1; j <= P; ++j) {
@@ -597,12 +598,12 @@ __global__ void k_fft_init(cx_t<T>* tw, T* sigma, T* dsym, int n, double h, int 
             }
             for (int j = 1; j <= dd_reach1(P); ++j) ds += dd_d1(P, j) * sinpi(2.0 * j * t / n);
             sigma[t] = (T)(4.0 * sg / (dd_d2den(P) * h * h));
-            dsym[t] = (T)(2.0 * ds / (dd_d1den(P) * h));
+            if (dsym) dsym[t] = (T)(2.0 * ds / (dd_d1den(P) * h));
         } else {
             const double s = sinpi((double)t / n);
             const double s2 = s * s;
             sigma[t] = (T)(4.0 * s2 * (3.0 + s2) * (1.0 / (3.0 * h * h)));
-            dsym[t] = (T)((8.0 * sinpi(2.0 * t / n) - sinpi(4.0 * t / n)) * (1.0 / (6.0 * h)));
+            if (dsym) dsym[t] = (T)((8.0 * sinpi(2.0 * t / n) - sinpi(4.0 * t / n)) * (1.0 / (6.0 * h)));
         }
     }
     pdl_trigger();
@@ -717,10 +718,11 @@ int setup_all() {
 
 template <typename T>
 int plan_init_t(PoissonPlan& p, const Geom& g, cudaStream_t s) {
-    if (device_malloc(&p.tw, sizeof(cx_t<T>) * p.n) != cudaSuccess) return -1;
+    constexpr bool fp32 = std::is_same<T, float>::value;
+    if (fp32 && device_malloc(&p.tw, sizeof(cx_t<T>) * p.n) != cudaSuccess) return -1;
     if (device_malloc(&p.ptw, sizeof(cx_t<T>) * 2 * p.n) != cudaSuccess) return -1;
     if (device_malloc(&p.sigma, sizeof(T) * p.n) != cudaSuccess) return -1;
-    if (device_malloc(&p.dsym, sizeof(T) * p.n) != cudaSuccess) return -1;
+    if (fp32 && device_malloc(&p.dsym, sizeof(T) * p.n) != cudaSuccess) return -1;
     if (setup_all<T>() != 0) return -2;
     { launch_pdl(k_fft_init<T>, (p.n + 255) / 256, 256, 0, s, (cx_t<T>*)p.tw, (T*)p.sigma, (T*)p.dsym, p.n,
                                                        g.h, g.P); note_launch(); }

@@ -69,10 +69,10 @@ void launch_ghost_rows(const int* list, int J, int* lat2idx, int* row_len, int* 
 struct PoissonPlan {
     int n = 0, logn = 0;
     bool fp32 = false;
-    void* tw = nullptr;      // exp(-2 pi i t/n), t < n (complex of the run's bulk type)
-    void* ptw = nullptr;     // the same twiddles as per-pass tables (see fft.cu)
+    void* tw = nullptr;      // FP32: exp(-2 pi i t/n), t < n
+    void* ptw = nullptr;     // the twiddles as per-pass tables (see fft.cu and fft_fixed.cuh)
     void* sigma = nullptr;   // symbol of the 4th-order second-derivative stencil
-    void* dsym = nullptr;    // symbol of the 4th-order first-derivative stencil (imaginary part)
+    void* dsym = nullptr;    // FP32: symbol of the 4th-order first-derivative stencil (imaginary part)
     void* inv = nullptr;     // FP64: 1/(n^2 (sigma(kx) + sigma(ky))), kx <= n/2 (see fft_fixed.cuh)
 };
 // 0, or -1 where the device memory for its tables cannot be had, or below.

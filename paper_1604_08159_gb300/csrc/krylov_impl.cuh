@@ -1,9 +1,10 @@
 #pragma once
 // Device helpers shared by the kernels of the Krylov projection (Sec. 2.1):
-// grid barriers with bounded waits, reductions in a fixed order, and phi_1 of
-// the projected system.  The vorticity form's kernels are in krylov_mma.cuh
-// and krylov_stream.cuh, the Rosenbrock step's in rosenbrock.cu, the
-// velocity-Exner form's in exner.cu.
+// the grid barrier with bounded waits, sums of a warp's lanes in a fixed
+// order, phi_1 of the projected system, and the end of a clustered launch.
+// The kernels are in krylov_mma.cuh and krylov_stream.cuh (digit products:
+// the vorticity form, and the velocity-Exner form while it fits), exner.cu
+// (its kernel with FP64 dots) and rosenbrock.cu.
 // On this part one warp issues at most one FP64 instruction per ~64 cycles
 // (about one per 16 cycles per SM), so what uses them is organised around the
 // count of FP64 instructions each warp issues.
@@ -20,51 +21,17 @@ namespace wrc {
 
 namespace {
 
-constexpr int kPT = 128;      // threads per block of the single-run kernel
+constexpr int kPT = 128;      // threads of the block that evaluates phi_1 for the Rosenbrock step
 constexpr int kNV = 32;       // accumulator slots: basis vectors per pass (<= m + 1 <= 32)
 constexpr int kOutP = 66;     // partial sums per block: two sets of (kNV dots + one product)
-constexpr int kGhostLanes = 8;   // lanes per ghost value (ghost_values, ghost_step)
+constexpr int kGhostLanes = 8;   // lanes per ghost value
 constexpr int kGatherLane = 8;   // row terms per lane fetched ahead of their additions
 static_assert(kGhostLanes * kGatherLane == kGhostRowMax, "one gather pass covers a whole interpolation row");
-constexpr int kCacheGroups = 16; // ghosts per block whose interpolation rows are kept in shared memory
-
-// Shared-memory copy of the interpolation rows of a block's first
-// kCacheGroups ghosts (ghost bid + nb q in slot q).
-struct RowCache {
-    int* len;
-    int* idx;      // kCacheGroups x kGhostRowMax
-    double* w;
-};
 
 __device__ __forceinline__ unsigned long long gtimer() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
-}
-
-// Calls f(std::integral_constant<int, t>) for t = n-1, n-2, ..., 0 (0 <= n <= N
-// <= 32): one jump into an unrolled sequence, so that the calls with t >= n
-// issue no instructions at all.  (A loop "if (t < n)" over all N unrolled
-// iterations becomes predicated instructions, and a predicated-off FP64
-// instruction still takes its ~64 issue cycles on this part; a "break" in the
-// loop keeps it from being unrolled, sending indexed accumulators to local
-// memory.)
-template <int N, typename F>
-__device__ __forceinline__ void down_from(int n, F&& f) {
-    static_assert(N >= 1 && N <= 32, "down_from covers at most 32 calls");
-    switch (n) {
-#define WRC_DOWN(t)                                            \
-    case (t) + 1:                                              \
-        if constexpr ((t) < N) f(std::integral_constant<int, (t)>{}); \
-        [[fallthrough]];
-        WRC_DOWN(31) WRC_DOWN(30) WRC_DOWN(29) WRC_DOWN(28) WRC_DOWN(27) WRC_DOWN(26) WRC_DOWN(25) WRC_DOWN(24)
-        WRC_DOWN(23) WRC_DOWN(22) WRC_DOWN(21) WRC_DOWN(20) WRC_DOWN(19) WRC_DOWN(18) WRC_DOWN(17) WRC_DOWN(16)
-        WRC_DOWN(15) WRC_DOWN(14) WRC_DOWN(13) WRC_DOWN(12) WRC_DOWN(11) WRC_DOWN(10) WRC_DOWN(9) WRC_DOWN(8)
-        WRC_DOWN(7) WRC_DOWN(6) WRC_DOWN(5) WRC_DOWN(4) WRC_DOWN(3) WRC_DOWN(2) WRC_DOWN(1) WRC_DOWN(0)
-#undef WRC_DOWN
-        default:
-            break;
-    }
 }
 
 // Sum of x over the 32 lanes of a warp, returned to every lane, through 40
@@ -151,164 +118,6 @@ __device__ bool grid_sync(unsigned* bar, int* err, unsigned long long limit_ns, 
     }
     __syncthreads();
     return (*(volatile int*)err & kErrStop) == 0;
-}
-
-// Per-block sums of acc[0..ndots) into dst[0..ndots) and, with NORM, of
-// acc[kNV] (a squared norm) into dst[ndots].  The first NS dot accumulators
-// (NS = ndots rounded up to a power of two) are reduced across the warp by a
-// reduce-scatter (NS - 1 exchanges; afterwards lane l holds the warp sum of
-// accumulator l mod NS), the norm by a shuffle tree.  Every FP64 addition
-// costs a warp ~64 cycles of issue on this part, so only the NS accumulators
-// in use take part.
-template <int PT, bool NORM>
-__device__ __forceinline__ void block_partials(double (&acc)[kNV + 1], int ndots, double* dst,
-                                               double (*s_red)[kNV + 1]) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (ndots > 0) {
-        int ns = 1;
-        while (ns < ndots) ns <<= 1;
-#pragma unroll
-        for (int s = 16; s >= 1; s >>= 1) {
-            if (2 * s > ns) continue;
-            const bool up = (lane & s) != 0;
-#pragma unroll
-            for (int i = 0; i < s; ++i) {
-                const double send = up ? acc[i] : acc[i + s];
-                const double keep = up ? acc[i + s] : acc[i];
-                acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-            }
-        }
-        for (int s = ns; s < 32; s <<= 1) acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], s);
-        if (lane < ns) s_red[wid][lane] = acc[0];
-    }
-    if (NORM) {
-        double v = acc[kNV];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) s_red[wid][kNV] = v;
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < ndots + (NORM ? 1 : 0); t += blockDim.x) {
-        const int src = t < ndots ? t : kNV;
-        double sum = 0.0;
-        for (int q = 0; q < PT / 32; ++q) sum += s_red[q][src];
-        dst[t] = sum;
-    }
-}
-
-// Sum over all blocks of part[b * kOutP + t], t < nout (<= 64), into s_out.
-// Up to 32 outputs, the lanes of a warp are split into L = 32 / ns groups
-// (ns = nout rounded up to a power of two, so L > 1 only for 16 outputs or
-// fewer): lane g ns + t of
-// warp w adds output t of blocks w + 4 (g + L u), u = 0, 1, ... (for 4 warps),
-// in order; the groups are then combined by shuffles and the warps' sums
-// added in warp order.  Same order in every block.  A lane's loads go out
-// kReduceBatch at a time ahead of their ordered additions, so one L2 round
-// trip covers up to kReduceBatch partials per lane; the additions of a
-// partial batch are entered by one jump (down_from: last partial first).  The partials were written by
-// other blocks before the grid barrier, whose fences make plain loads see
-// them (L1 is invalidated there).
-constexpr int kReduceBatch = 24;
-
-template <int PT>
-__device__ __forceinline__ void reduce_all(const double* part, int nout, double* s_out,
-                                           double (*s_red)[kNV + 1], int nb) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int kW = PT / 32;
-    if (nout > 32) {
-        // two chunks: lane t adds outputs t and 32 + t (if any) of blocks
-        // w, w + 4, ..., the loads of both going out together
-        constexpr int kB = kReduceBatch / 2;
-        const int t2 = 32 + lane;
-        const bool has2 = t2 < nout;
-        double v1 = 0.0, v2 = 0.0;
-        const double* p = part + lane;
-        int b = wid;
-        for (; b + (kB - 1) * kW < nb; b += kB * kW) {
-            double x1[kB], x2[kB];
-#pragma unroll
-            for (int u = 0; u < kB; ++u) {
-                x1[u] = p[(size_t)(b + u * kW) * kOutP];
-                x2[u] = has2 ? p[32 + (size_t)(b + u * kW) * kOutP] : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < kB; ++u) {
-                v1 += x1[u];
-                v2 += x2[u];
-            }
-        }
-        const int rest = b < nb ? (nb - 1 - b) / kW + 1 : 0;   // < kB
-        double x1[kB], x2[kB];
-#pragma unroll
-        for (int u = 0; u < kB; ++u)
-            if (u < rest) {
-                x1[u] = p[(size_t)(b + u * kW) * kOutP];
-                x2[u] = has2 ? p[32 + (size_t)(b + u * kW) * kOutP] : 0.0;
-            }
-        down_from<kB>(rest, [&](auto uc) {
-            constexpr int u = decltype(uc)::value;
-            v1 += x1[u];
-            v2 += x2[u];
-        });
-        s_red[wid][lane] = v1;
-        __syncthreads();
-        for (int q = threadIdx.x; q < 32; q += blockDim.x) {
-            double sum = 0.0;
-            for (int w = 0; w < kW; ++w) sum += s_red[w][q];
-            s_out[q] = sum;
-        }
-        __syncthreads();
-        s_red[wid][lane] = v2;
-        __syncthreads();
-        for (int q = threadIdx.x; q < nout - 32; q += blockDim.x) {
-            double sum = 0.0;
-            for (int w = 0; w < kW; ++w) sum += s_red[w][q];
-            s_out[32 + q] = sum;
-        }
-        __syncthreads();
-        return;
-    }
-    int ns = 1;
-    while (ns < nout) ns <<= 1;
-    const int L = 32 / ns;
-    const int t = lane & (ns - 1), g = lane / ns;
-    const int bstep = kW * L;
-    double v = 0.0;
-    if (t < nout) {
-        const double* p = part + t;
-        int b = wid + kW * g;
-        for (; b + (kReduceBatch - 1) * bstep < nb; b += kReduceBatch * bstep) {
-            double x[kReduceBatch];
-#pragma unroll
-            for (int u = 0; u < kReduceBatch; ++u) x[u] = p[(size_t)(b + u * bstep) * kOutP];
-#pragma unroll
-            for (int u = 0; u < kReduceBatch; ++u) v += x[u];
-        }
-        const int rest = b < nb ? (nb - 1 - b) / bstep + 1 : 0;   // < kReduceBatch
-        double x[kReduceBatch];
-#pragma unroll
-        for (int u = 0; u < kReduceBatch; ++u)
-            if (u < rest) x[u] = p[(size_t)(b + u * bstep) * kOutP];
-        down_from<kReduceBatch>(rest, [&](auto uc) { v += x[decltype(uc)::value]; });
-    }
-    // the L groups, added in group order by the lanes of group 0 (shared
-    // memory rather than a shuffle tree: see warp_sum)
-    s_red[wid][lane] = v;
-    __syncwarp();
-    if (L > 1) {
-        double c = v;
-        if (g == 0 && t < nout)
-            for (int q = 1; q < L; ++q) c += s_red[wid][q * ns + t];
-        __syncwarp();
-        if (g == 0 && t < nout) s_red[wid][t] = c;
-    }
-    __syncthreads();
-    for (int q = threadIdx.x; q < nout; q += blockDim.x) {
-        double sum = 0.0;
-        for (int w = 0; w < kW; ++w) sum += s_red[w][q];
-        s_out[q] = sum;
-    }
-    __syncthreads();
 }
 
 // ---- phi_1 from the exponential of the augmented matrix ------------------
@@ -452,35 +261,12 @@ __device__ __forceinline__ double f2d_exact(float x) {
 __device__ __forceinline__ double dbl(double x) { return x; }
 __device__ __forceinline__ double dbl(float x) { return f2d_exact(x); }
 
-// sqrt(q) and 1/sqrt(q) in FP64 for the normalisation of a new basis vector:
-// an FP32 reciprocal square root as the seed, then two Newton-Raphson steps
-// y <- y (3/2 - (q/2) y^2) in FP64 (each doubles the correct bits: ~22 -> ~44
-// -> full precision), sqrt(q) = q y; three dependent FP64 operations per
-// step.  FP64 division and square root are long instruction sequences on
-// this part.  q outside [2^-99, 2^99] (or negative, or not finite) takes the
-// library's sqrt and division; the range test is integer work on the
-// exponent.
-__device__ __forceinline__ void sqrt_and_rsqrt(double q, double& s, double& r) {
-    const int hi = __double2hiint(q);
-    const int e = (hi >> 20) & 0x7ff;
-    if (hi >= 0 && e > 1023 - 99 && e < 1023 + 99) {
-        const double hq = 0.5 * q;
-        double y = (double)rsqrtf((float)q);
-        y = y * fma(-hq, y * y, 1.5);
-        y = y * fma(-hq, y * y, 1.5);
-        r = y;
-        s = q * y;
-    } else {
-        s = sqrt(q);
-        r = 1.0 / s;
-    }
-}
-
-// End of a clustered launch: wait for the second barrier of the last
-// step_dots call (if there was one), then take part in the cluster barriers
-// of the calls this block did not make (a breakdown, a failed grid barrier,
-// a refusal), so that every block of a cluster passes exactly 2m cluster
-// barriers and none exits while a peer may still read its shared memory.
+// End of a clustered launch of m Arnoldi steps' dots, `calls` of which this
+// block has taken: wait for the second cluster barrier of the last of them
+// (if there was one), then take part in the barriers of those it did not take
+// (a breakdown, a failed grid barrier, a refusal), so that every block of a
+// cluster passes exactly 2 m of them and none exits while a peer may still
+// read its shared memory.
 // (Only for a launch that formed its clusters.)
 // Each of these waits ends: every block of the cluster reaches its own
 // remaining barriers, all its grid-barrier waits being bounded.

@@ -21,10 +21,13 @@
 //    joined in integers;
 //  - basis vectors: |q| <= 1, so one fixed scale, 2^-61 per unit; u and z:
 //    a scale per block (its largest value's exponent); s and t: one scale.
-//    A product is kept to 2^-61 of the largest one, finer than the rounding
-//    of an FP64 running sum over the same points; sums across warps, blocks
-//    and the grid are integer additions, hence exact and independent of
-//    their order.
+//    The digit products beyond the eighth column are left out: a sum over
+//    n points is off by less than n 2^-58 of the largest product (2^-61 a
+//    product, root mean square), finer in norm than the rounding of an FP64
+//    running sum over the same points, though not for every single entry.
+//    Sums across warps, blocks and the grid are integer additions, exact and
+//    independent of their order; how the points are dealt over blocks, whose
+//    scales differ, still shows in the last bits.
 // Layout: a block owns grid points and its share of the ghosts as columns of
 // a table [row of the basis][column] in shared memory, as digits (halves) or
 // as 64-bit integers whose digits are unpacked while they are loaded, so
@@ -127,14 +130,6 @@ __device__ __forceinline__ void digits2(unsigned x, unsigned y, int q, unsigned&
     const unsigned p = __byte_perm(x, y, q == 0 ? 0x6273 : 0x4051);
     d0 = unbias2(__byte_perm(p, 0x64646464u, 0x4140));
     d1 = unbias2(__byte_perm(p, 0x64646464u, 0x4342));
-}
-// The eight digits of two 64-bit numbers, most significant first.
-__device__ __forceinline__ void digits8(unsigned long long x, unsigned long long y, unsigned (&d)[8]) {
-    const unsigned xh = (unsigned)(x >> 32), yh = (unsigned)(y >> 32), xl = (unsigned)x, yl = (unsigned)y;
-    digits2(xh, yh, 0, d[0], d[1]);
-    digits2(xh, yh, 1, d[2], d[3]);
-    digits2(xl, yl, 0, d[4], d[5]);
-    digits2(xl, yl, 1, d[6], d[7]);
 }
 // One 64-bit number's digits as halves into a tile: digit i at row i.
 __device__ __forceinline__ void put_digits(char* at, int pitch, unsigned long long x) {
@@ -747,10 +742,11 @@ __device__ __forceinline__ void put_value(char* Qb, int pitch, int dstride, int 
 // ---- q_j and the next u at one column ------------------------------------------
 // q_j = (u - ps) / h, next u = (z - pc - q_j qz) / h with ps = sum s_t q_t and
 // pc = sum t_t q_t as exact integers (vs 2^es, vt 2^et).  FP64: one rounding
-// per operation.  Mixed mode: u - ps and the results are FP32; the second
-// value is formed in FP32 pairs (exact products by fma, exact sums), whose
-// ~2^-45 stays far below the FP32 rounding of the result: FP64 instructions
-// would cost 65 cycles each here.
+// per operation.  Mixed mode: ps and pc are rounded to FP32 (2^-24 of
+// them, as coefficients and sums of this mode are), u - ps and the results
+// are FP32, and z - pc - q_j qz is formed in FP32 pairs (exact products by fma,
+// exact sums), so that its cancellation adds nothing of its own: FP64
+// instructions would cost 65 cycles each here.
 struct StepScalars {
     double hinv, qz;
     float hh, hl, qh, ql;   // the same two as FP32 pairs

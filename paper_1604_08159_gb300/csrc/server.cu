@@ -151,9 +151,9 @@ int64_t run_steps(wrc_run* R) {
     return stats[1];
 }
 
-// Block shape of one batched step of `runs`: the server's, else the
-// autotuned one for this precision and size, else 128 x 1; 64 threads when
-// more runs than co-resident blocks of the chosen shape.
+// Shape of one batched step of `runs`: the server's, else the autotuned one
+// for this precision and size, else 128 x 1; 64 when more runs than a batch of
+// the chosen one takes.
 void pick_shape(const wrc_server* S, BatchCtx& C, const std::vector<wrc_run*>& runs) {
     int pt = 128, ept = 1;
     if (S->cfg.threads_per_block > 0) {
