@@ -274,7 +274,7 @@ KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int d
 // The velocity-Exner step takes the same kernel while its 3 n entries fit
 // (up to ~30K points at m = 30): with two barriers per Arnoldi step instead of
 // the four and FP64 dots of k_ex_krylov, which runs what does not fit, a step
-// of 7.5K points at 1024^2, m = 30, takes 489 us instead of 1327.
+// of 8.6K points at 1024^2, m = 30, takes 486 us instead of 1318.
 KrylovPlan krylov_ex_plan(long long n, long long ng, int m, int P, int dev) {
     return krylov_plan(3 * n, 3 * ng, m, false, P, dev, 1);
 }
