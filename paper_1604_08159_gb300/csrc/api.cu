@@ -1982,9 +1982,10 @@ wrc_status plan_batch(BatchCtx& C, const std::vector<wrc_run*>& runs, int& total
         if (C.d_blk) cudaFree(C.d_blk);
         C.h_blk = nullptr;
         C.d_blk = nullptr;
+        C.blk_cap = 0;
+        BCK(cudaMallocHost((void**)&C.h_blk, sizeof(int) * (need + 1024)));
+        BCK(device_malloc((void**)&C.d_blk, sizeof(int) * (need + 1024)));
         C.blk_cap = need + 1024;
-        BCK(cudaMallocHost((void**)&C.h_blk, sizeof(int) * C.blk_cap));
-        BCK(cudaMalloc((void**)&C.d_blk, sizeof(int) * C.blk_cap));
     }
     if ((int)M > C.args_cap) {
         BCK(cudaStreamSynchronize(C.main));
@@ -1992,9 +1993,10 @@ wrc_status plan_batch(BatchCtx& C, const std::vector<wrc_run*>& runs, int& total
         if (C.d_args) cudaFree(C.d_args);
         C.h_args = nullptr;
         C.d_args = nullptr;
+        C.args_cap = 0;
+        BCK(cudaMallocHost((void**)&C.h_args, sizeof(KrylovStepArgs) * (M + 64)));
+        BCK(device_malloc((void**)&C.d_args, sizeof(KrylovStepArgs) * (M + 64)));
         C.args_cap = (int)M + 64;
-        BCK(cudaMallocHost((void**)&C.h_args, sizeof(KrylovStepArgs) * C.args_cap));
-        BCK(cudaMalloc((void**)&C.d_args, sizeof(KrylovStepArgs) * C.args_cap));
     }
     std::copy(items.begin(), items.end(), C.h_blk);
     std::copy(off.begin(), off.end(), C.h_blk + items.size());

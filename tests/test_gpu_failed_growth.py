@@ -95,3 +95,26 @@ def test_tables_of_the_solve(monkeypatch):
         run.init_vortices(VORT)
         run.step(1)
         run.sync()
+
+
+def test_tables_of_a_batched_launch(monkeypatch):
+    """The launch's block table refused at the first step: an error, and after a
+    new initial condition a step as if nothing had happened."""
+    prm = small_params()
+    ref = None
+    for refuse in (False, True):
+        with B.Ensemble([prm, prm]) as ens:
+            for mem in ens.members:
+                mem.init_vortices(VORT)
+            if refuse:
+                monkeypatch.setenv("WRC_ALLOC_TEST_LIMIT", "1000")
+                with pytest.raises(B.WrcError):
+                    ens.step(1)
+                monkeypatch.delenv("WRC_ALLOC_TEST_LIMIT")
+                for mem in ens.members:
+                    mem.init_vortices(VORT)
+            ens.step(1)
+            got = ens.members[1].active()
+            ref = ref or got
+            for x, y in zip(got, ref):
+                assert np.array_equal(x, y)
