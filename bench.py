@@ -569,7 +569,7 @@ KRYLOV_SOURCES = ("csrc/krylov_impl.cuh", "csrc/krylov_mma.cuh", "csrc/exner_op.
 # DRAM bytes per launch of the Krylov kernel on the 1024^2 pair, from one ncu
 # capture (dram__bytes_read.sum + dram__bytes_write.sum), valid only for the
 # kernel sources whose SHA-256 is recorded with it.
-KRYLOV_TRAFFIC = {"sources_sha256": "2f6706585f037936660e6a2aa05fe5d875d9035141cc9faa1b086016e5a14bfc",
+KRYLOV_TRAFFIC = {"sources_sha256": "78abbbd0f0b56af26e983639f7118b65e9daf7e7bbc3f797cf8fd3041cdde661",
                   "bytes_per_launch": 2539008,
                   "capture": "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum, 1024^2 pair, second launch"}
 

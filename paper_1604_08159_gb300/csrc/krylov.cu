@@ -197,15 +197,17 @@ int krylov_step_init(int dev, bool fp32, int P, int* max_blocks) {
 
 // Launch rule.  The kernel with its table in shared memory takes every problem
 // that fits one block per SM; beyond, the streaming one.  Points per
-// block: spread over all SMs, but at least 48 at order 4 and 32 above (the
-// higher orders' longer ghost rows queue for a block's few warps: 64 points
-// make a mixed run of 3-4K points 8-10% slower).  A block has its SM to itself, so
-// runs stepped at the same time, each on a stream of its own, share the
-// device only where their blocks leave SMs free.  48 points cost a run alone
-// nothing and let two small ones run side by side (128^2, 2.8K points, us a
-// step alone / each of four / each of eight at once: 603 / 166 / 90 with the
-// FP64 dots, 337 / 213 / 212 from 32 points on, 335 / 115 / 112 from 48, 345
-// / 100 / 82 from 64).  Larger runs keep all SMs, as half of them cost a run
+// block: spread over all SMs, but at least 32, and 48 for order-4 runs of up
+// to 3072 points.  A block has its SM to itself, so runs stepped at the same
+// time, each on a stream of its own, share the device only where their blocks
+// leave SMs free.  Up to 3072 points 48 a block cost a run alone nothing in
+// FP64, 2% of a step in the mixed mode, and let two work side by side (128^2, 2.8K
+// points, us a step alone / each of four / each of eight at once: 603 / 166 /
+// 90 with the FP64 dots, 337 / 213 / 212 from 32 points on, 335 / 115 / 112
+// so, 345 / 100 / 82 from 64).  Above, 32 points make more blocks than
+// clusters are formed for, 3-4% faster than 48 in clusters; at higher orders
+// longer ghost rows queue for a block's few warps (64 points: 8-10% slower
+// at 3-4K points).  Larger runs keep all SMs, as half of them cost a run
 // alone 3-10% (256^2, 9.2K points: 754 / 241 / 189, 445 / 294 / 297, on half
 // the SMs 472 / 181 / 180): alone they take 0.5 to 0.7 of the time with the
 // FP64 dots, four or eight at once up to 1.9 times it; an ensemble's one
@@ -228,7 +230,7 @@ KrylovPlan krylov_plan(long long n, long long ng, int m, bool fp32, int P, int d
     const auto up16 = [](long long x) { return (int)((x + 15) / 16 * 16); };
     {
         int ppb = up16((n + c.cap1 - 1) / std::max(1, c.cap1));
-        ppb = std::max(ppb, P == 2 ? 48 : 32);
+        ppb = std::max(ppb, P == 2 && n <= 3072 ? 48 : 32);
         int nb = (int)((n + ppb - 1) / ppb);
         nb = nb < 1 ? 1 : nb;
         int cl = 1;
