@@ -762,10 +762,9 @@ KrylovStepArgs krylov_args_scalar(wrc_run* R) {
 }
 
 // The Krylov steps of omega and of the passive scalar as two problems of one
-// cooperative launch of the batched kernel (each with half of the co-resident
-// blocks, its own grid barrier and workspace), so that the latency-bound
-// phases of one overlap the FP64 work of the other.  The scalar's workspace
-// grows with the grid here.
+// cooperative launch of the streaming kernel (each with half of the SMs, its
+// own grid barrier and workspace).  The scalar's workspace grows with the grid
+// here.
 template <typename T>
 wrc_status krylov_pair(wrc_run* R, const KrylovStepArgs& A) {
     const cudaStream_t s = R->st;
@@ -2401,7 +2400,7 @@ wrc_status wrc_ensemble_tune(wrc_ensemble* E, int32_t steps_per_candidate, int32
     batch_take_profile(E->C);
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 3; ++b) {
-            // a shape needs one co-resident block per member at least
+            // (a batch of a shape takes so many members at most)
             if (krylov_batch_max_runs(pts[a]) < (int)E->members.size()) continue;
             E->C.pt = pts[a];
             E->C.ept = epts[b];
